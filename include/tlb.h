@@ -217,9 +217,9 @@ long long tlb_launch_count(const tlb_ctx *ctx);
  * that cannot afford the device-wide synchronisation cudaMalloc/cudaFree may
  * imply.  tlb_step_noalloc advances caller-owned populations by nsteps with
  * the kernels of tlb_step (the same populations, bit for bit) and allocates
- * nothing: its scratch (moments, tile table, node flags, error word, the two
- * batch entries) is one static device array of TLB_NOALLOC_MAX_NODES * 25 +
- * 1280 bytes (26.2 MB) that every GPU loading this library holds until exit.
+ * nothing: its scratch (moments, node flags, wall-tile flags, error word) is
+ * one static device array of TLB_NOALLOC_MAX_NODES * 10 + 256 bytes (10.5 MB)
+ * that every GPU loading this library holds until exit.
  *   p          lattice, sizes and physics; at most TLB_NOALLOC_MAX_NODES
  *              (1048576) nodes, else TLB_E_INVAL; g_fp16 must be 0.  Force
  *              wetting given by angles takes its strengths from the
@@ -235,9 +235,8 @@ long long tlb_launch_count(const tlb_ctx *ctx);
  * The first call on a device looks up the scratch array's device address
  * (once per device, with that device current).  All calls share the one
  * array and it keeps the last call's contents.  Every call resets the error
- * word and rewrites the batch entries (they hold f, g and their work
- * buffers).  The node flags and the tile table are built on the host and
- * uploaded when the lattice, the sizes, the mask's contents or the
+ * word.  The node flags are built on the host and uploaded, and the wall-tile
+ * flags formed from them, when the lattice, the sizes, the mask's contents or the
  * stream differ from the previous call's on this device; otherwise the copy
  * in the array is used again (one N-byte comparison instead of the host pass
  * over the mask and its upload).  Calls that overlap on the GPU --

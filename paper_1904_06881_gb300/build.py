@@ -32,9 +32,14 @@ BUILD_TIMEOUT = os.path.join(HERE, "_build_timeout")
 LIB_TIMEOUT = os.path.join(BUILD_TIMEOUT, "libtlb.so")
 ROOT = os.path.dirname(HERE)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--use_fast_math", "-diag-suppress", "177"]
+# Approximate division and square root, denormals flushed; multiply-adds are
+# contracted only where the source says fmaf, so that one function gives the
+# same bits in every kernel and build it is inlined into (a lattice alone and in
+# a batch, the checked build, the one- and two-kernel D3Q27 step).
+FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-ftz=true", "-prec-div=false", "-prec-sqrt=false",
+         "-fmad=false", "-diag-suppress", "177"]
 SOURCES = ["tlb_api.cu", "tlb_d2q9.cu", "tlb_d3q27.cu"]
-HEADERS = ["tlb_device.cuh", "tlb_kernels.cuh", "tlb_internal.h"]
+HEADERS = ["tlb_device.cuh", "tlb_kernels.cuh", "tlb_step.cuh", "tlb_internal.h"]
 
 
 def _nvcc():

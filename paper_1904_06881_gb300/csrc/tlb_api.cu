@@ -393,12 +393,14 @@ static DevParams make_dev(const tlb_params &p, const tlb_derived &d)
     q.nz = p.nz;
     q.N = (long long)p.nx * p.ny * p.nz;
     q.lam1 = (float)p.lambda[0];
+    q.hl1 = (float)(0.5 * p.lambda[0]);
     q.lam2 = (float)p.lambda[1];
     q.lam3 = (float)p.lambda[2];
     q.chi = (float)p.chi;
     q.inv_chi = (float)(1.0 / p.chi);
     q.a = (float)d.a;
     q.b = (float)d.b;
+    q.b4 = (float)(d.b / 4.0);
     q.RT = (float)(d.R * d.T);
     q.C = (float)d.C;
     q.Psi0 = (float)d.Psi0;
@@ -448,11 +450,10 @@ struct tlb_ctx {
     long long steps = 0;
     long long launches = 0;
     int sticky = TLB_OK;
-    // the lattice as a batch of one: entries for both buffer parities, tile table
     CUtensorMap *tmaps = nullptr;     // D3Q27: per parity, tensor maps of f_in and g_in (null if unused)
-    BatchEntry *self_entries = nullptr;
-    int4 *self_tiles = nullptr;
-    int nself_tiles = 0;
+    uint8_t *wall_tiles = nullptr;    // per tile: 1 with a solid node within two links
+    uint32_t wall_bits[WALL_WORDS] = {};   // the same as bits (lattices of few tiles)
+    int wall_known = 0;
     // one CUDA graph per buffer parity holding the launches of a step (D3Q27)
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     cudaStream_t cap_stream = nullptr;
@@ -585,10 +586,24 @@ static bool encode_tensor_maps(const tlb_ctx *c, CUtensorMap maps[6])
     return true;
 }
 
-// the entry's tensor-map pointers for input buffer `cur` (all null without maps)
-static void entry_maps(const tlb_ctx *c, int cur, BatchEntry &e)
+// the lattice as the stepping kernels take it, reading population buffer `cur`
+static BatchEntry make_entry(const tlb_ctx *c, int cur)
 {
+    BatchEntry e = {};
+    e.p = c->dp;
+    e.f_in = c->s.f[cur];
+    e.f_out = c->s.f[1 - cur];
+    e.g_in = c->s.g[cur];
+    e.g_out = c->s.g[1 - cur];
+    e.rho = c->s.rho;
+    e.phi = c->s.phi;
+    e.type = c->s.type;
+    e.status = c->s.status;
     for (int k = 0; k < 3; ++k) e.tm[k] = c->tmaps ? (const void *)(c->tmaps + 3 * cur + k) : nullptr;
+    e.wall_tiles = c->wall_tiles;
+    e.wall_known = c->wall_known;
+    std::memcpy(e.wall_bits, c->wall_bits, sizeof(e.wall_bits));
+    return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -748,34 +763,10 @@ extern "C" int tlb_create_ex(const tlb_params *pin, tlb_ctx **out)
         }
     }
     {
-        // batch-of-one tables: entry per buffer parity, one tile per CTA
-        int D = c->D;
-        int TX = D == 2 ? Launch<2>::tile_dims(0) : Launch<3>::tile_dims(0);
-        int TY = D == 2 ? Launch<2>::tile_dims(1) : Launch<3>::tile_dims(1);
-        int TZ = D == 2 ? Launch<2>::tile_dims(2) : Launch<3>::tile_dims(2);
-        std::vector<int4> tiles;
-        for (int z = 0; z < c->p.nz; z += TZ)
-            for (int y = 0; y < c->p.ny; y += TY)
-                for (int x = 0; x < c->p.nx; x += TX) tiles.push_back(make_int4(0, x, y, z));
-        BatchEntry ent[2];
-        for (int par = 0; par < 2; ++par) {
-            ent[par].p = c->dp;
-            ent[par].f_in = c->s.f[par];
-            ent[par].f_out = c->s.f[1 - par];
-            ent[par].g_in = c->s.g[par];
-            ent[par].g_out = c->s.g[1 - par];
-            ent[par].rho = c->s.rho;
-            ent[par].phi = c->s.phi;
-            ent[par].type = c->s.type;
-            ent[par].status = c->s.status;
-            entry_maps(c, par, ent[par]);
-        }
-        ALLOC_LATE(c->self_entries, sizeof(ent));
-        ALLOC_LATE(c->self_tiles, tiles.size() * sizeof(int4));
-        c->nself_tiles = (int)tiles.size();
-        cudaMemcpyAsync(c->self_entries, ent, sizeof(ent), cudaMemcpyHostToDevice, c->stream);
-        cudaMemcpyAsync(c->self_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, c->stream);
-        cudaStreamSynchronize(c->stream);
+        const size_t nt = (size_t)(c->D == 2 ? Launch<2>::tiles(c->dp) : Launch<3>::tiles(c->dp));
+        ALLOC_LATE(c->wall_tiles, nt);
+        cudaMemsetAsync(c->wall_tiles, 0, nt, c->stream);
+        c->wall_known = nt <= 32 * WALL_WORDS;         // no walls yet
     }
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
@@ -913,6 +904,17 @@ extern "C" int tlb_set_solid(tlb_ctx *c, const uint8_t *mask)
         c->ghosts_cap = ng;
     }
     if (ng) CUDA_TRY(cudaMemcpyAsync(c->ghosts_dev, c->ghost_host.data(), ng * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    DISPATCH(c, wall_tiles(c->dp, c->s.type, c->wall_tiles, c->stream));
+    CUDA_TRY(cudaGetLastError());
+    if (c->wall_known) {
+        const int nt = c->D == 2 ? Launch<2>::tiles(c->dp) : Launch<3>::tiles(c->dp);
+        uint8_t w[32 * WALL_WORDS];
+        CUDA_TRY(cudaMemcpyAsync(w, c->wall_tiles, (size_t)nt, cudaMemcpyDeviceToHost, c->stream));
+        CUDA_TRY(cudaStreamSynchronize(c->stream));
+        std::memset(c->wall_bits, 0, sizeof(c->wall_bits));
+        for (int k = 0; k < nt; ++k)
+            if (w[k]) c->wall_bits[k >> 5] |= 1u << (k & 31);
+    }
     c->s.ghosts = c->ghosts_dev;
     c->s.nghost = (int)ng;
     CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -953,7 +955,7 @@ static int init_from_device(tlb_ctx *c, const float *u_dev)
 {
     DISPATCH(c, ghosts(c->dp, c->s, c->stream));
     AuxOut none = {};
-    DISPATCH(c, step(c->dp, c->s, MODE_INIT, u_dev, none, c->stream));
+    DISPATCH(c, field_pass(c->dp, c->s, MODE_INIT, u_dev, none, c->stream));
     c->steps = 0;
     return check_launch(c, 2);
 }
@@ -1007,18 +1009,17 @@ extern "C" int tlb_init_fields(tlb_ctx *c, const double *rho, const double *phi,
 // moments it needs), D3Q27 two (moments, step).
 static int launches_per_step(int D) { return D == 2 ? 1 : 2; }
 
-// The launches of one step of a lattice, as a batch of one (the kernels
-// tlb_step_batch uses, so alone and batched results are bit-identical).
-// Phase 0 is the moments pass (D3Q27 only), phase 2 the step kernel.
+// The launches of one step of a lattice alone (the tile code of the batched
+// kernels, so alone and batched results are bit-identical).  Phase 0 is the
+// moments pass (D3Q27 only), phase 2 the step kernel.
 static void issue_phase(tlb_ctx *c, int phase, cudaStream_t st)
 {
-    const BatchEntry *E = c->self_entries + c->s.cur;
-    int fp16 = c->p.g_fp16;
+    const BatchEntry e = make_entry(c, c->s.cur);
     if (c->D == 2) {
-        if (phase == 2) Launch<2>::step_batch(E, c->self_tiles, c->nself_tiles, fp16, st);
+        if (phase == 2) Launch<2>::step(e, st);
     } else {
-        if (phase == 0) Launch<3>::moments_batch(E, c->self_tiles, c->nself_tiles, fp16, st);
-        else if (phase == 2) Launch<3>::step_batch(E, c->self_tiles, c->nself_tiles, fp16, st);
+        if (phase == 0) Launch<3>::moments_step(e, st);
+        else if (phase == 2) Launch<3>::step(e, st);
     }
 }
 
@@ -1173,7 +1174,7 @@ extern "C" int tlb_get_aux(tlb_ctx *c, int which, double *out)
         else if (which == 2) a.mup = dst;
         else if (which <= 5) a.F[which - 3] = dst;
         else a.P[which - 6] = dst;
-        DISPATCH(c, step(c->dp, c->s, MODE_AUX, nullptr, a, c->stream));
+        DISPATCH(c, field_pass(c->dp, c->s, MODE_AUX, nullptr, a, c->stream));
         ++nl;
         src = dst;
     }
@@ -1294,6 +1295,13 @@ struct BatchPlan {
     int ntiles = 0;
 };
 
+static bool any_big(const std::vector<tlb_ctx *> &ctxs)
+{
+    for (const tlb_ctx *c : ctxs)
+        if (big_lattice(c->N)) return true;
+    return false;
+}
+
 static int build_plan(tlb_ctx *const *ctxs, int n, BatchPlan &plan, cudaStream_t st)
 {
     int D = ctxs[0]->D;
@@ -1307,18 +1315,7 @@ static int build_plan(tlb_ctx *const *ctxs, int n, BatchPlan &plan, cudaStream_t
         if (c->D != D) return fail(TLB_E_INVAL, "batched lattices must share the lattice type");
         if (c->p.g_fp16 != ctxs[0]->p.g_fp16) return fail(TLB_E_INVAL, "batched lattices must share the g storage");
         for (int par = 0; par < 2; ++par) {
-            BatchEntry &e = par ? e1[k] : e0[k];
-            int cur = (c->s.cur + par) & 1;
-            e.p = c->dp;
-            e.f_in = c->s.f[cur];
-            e.f_out = c->s.f[1 - cur];
-            e.g_in = c->s.g[cur];
-            e.g_out = c->s.g[1 - cur];
-            e.rho = c->s.rho;
-            e.phi = c->s.phi;
-            e.type = c->s.type;
-            e.status = c->s.status;
-            entry_maps(c, cur, e);
+            (par ? e1[k] : e0[k]) = make_entry(c, (c->s.cur + par) & 1);
         }
         for (int z = 0; z < c->p.nz; z += TZ)
             for (int y = 0; y < c->p.ny; y += TY)
@@ -1347,10 +1344,10 @@ static int run_plan(BatchPlan &plan, int nsteps, cudaStream_t st)
         const BatchEntry *E = plan.entries[s & 1];
         int fp16 = plan.ctxs[0]->p.g_fp16;
         if (D == 2) {
-            Launch<2>::step_batch(E, plan.tiles, plan.ntiles, fp16, st);
+            Launch<2>::step_batch(E, plan.tiles, plan.ntiles, fp16, any_big(plan.ctxs), st);
         } else {
             Launch<3>::moments_batch(E, plan.tiles, plan.ntiles, fp16, st);
-            Launch<3>::step_batch(E, plan.tiles, plan.ntiles, fp16, st);
+            Launch<3>::step_batch(E, plan.tiles, plan.ntiles, fp16, false, st);
         }
     }
     cudaError_t e = cudaGetLastError();
@@ -1450,18 +1447,7 @@ static int batch_write_entries(tlb_batch *b)
         tlb_ctx *c = b->ctxs[k];
         b->base_cur[k] = c->s.cur;
         for (int par = 0; par < 2; ++par) {
-            BatchEntry &x = e[par][k];
-            int cur = (c->s.cur + par) & 1;
-            x.p = c->dp;
-            x.f_in = c->s.f[cur];
-            x.f_out = c->s.f[1 - cur];
-            x.g_in = c->s.g[cur];
-            x.g_out = c->s.g[1 - cur];
-            x.rho = c->s.rho;
-            x.phi = c->s.phi;
-            x.type = c->s.type;
-            x.status = c->s.status;
-            entry_maps(c, cur, x);
+            e[par][k] = make_entry(c, (c->s.cur + par) & 1);
         }
     }
     for (int par = 0; par < 2; ++par)
@@ -1483,10 +1469,10 @@ static void batch_issue(const tlb_batch *b, int par, cudaStream_t st)
 {
     const BatchEntry *E = b->entries[par];
     if (b->D == 2) {
-        Launch<2>::step_batch(E, b->tiles, b->ntiles, b->fp16, st, b->cfg.variant);
+        Launch<2>::step_batch(E, b->tiles, b->ntiles, b->fp16, any_big(b->ctxs), st, b->cfg.variant);
     } else {
         Launch<3>::moments_batch(E, b->tiles, b->ntiles, b->fp16, st);
-        Launch<3>::step_batch(E, b->tiles, b->ntiles, b->fp16, st, b->cfg.variant);
+        Launch<3>::step_batch(E, b->tiles, b->ntiles, b->fp16, false, st, b->cfg.variant);
     }
 }
 
@@ -2013,15 +1999,13 @@ extern "C" void tlb_server_destroy(tlb_server *s)
 // live in one file-scope device array, so the call performs no cudaMalloc,
 // cudaFree or other allocation on the device.
 // ---------------------------------------------------------------------------
-// layout, M = TLB_NOALLOC_MAX_NODES: rho (M floats) | phi (M floats) |
-// tiles (M int4: a tile holds at least one node) | flags (M bytes) |
-// status word (256 bytes reserved) | entries (2 BatchEntry, 1024 bytes reserved)
+// layout, M = TLB_NOALLOC_MAX_NODES: rho (M floats) | phi (M floats) | flags (M
+// bytes) | wall tiles (M bytes: a tile holds at least one node) | status word
+// (256 bytes reserved)
 constexpr size_t NOALLOC_M = TLB_NOALLOC_MAX_NODES;
-constexpr size_t NOALLOC_PHI = NOALLOC_M * 4, NOALLOC_TILES = NOALLOC_M * 8, NOALLOC_FLAGS = NOALLOC_M * 24,
-                 NOALLOC_STATUS = NOALLOC_M * 25, NOALLOC_ENTRIES = NOALLOC_M * 25 + 256,
-                 NOALLOC_BYTES = NOALLOC_M * 25 + 256 + 1024;
-static_assert(2 * sizeof(BatchEntry) <= 1024, "batch entries exceed their reserved bytes");
-static_assert(NOALLOC_TILES % 16 == 0 && NOALLOC_ENTRIES % 256 == 0, "scratch alignment");
+constexpr size_t NOALLOC_PHI = NOALLOC_M * 4, NOALLOC_FLAGS = NOALLOC_M * 8, NOALLOC_WALLS = NOALLOC_M * 9,
+                 NOALLOC_STATUS = NOALLOC_M * 10, NOALLOC_BYTES = NOALLOC_M * 10 + 256;
+static_assert(NOALLOC_STATUS % 256 == 0, "scratch alignment");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
 namespace {
@@ -2031,7 +2015,7 @@ struct NoallocDevice {
     // the geometry whose node flags and ghost list the array holds, and the
     // stream that uploaded them (later work on that stream sees the upload)
     bool have_geom = false;
-    int lattice = -1, nx = 0, ny = 0, nz = 0, ntiles = 0;
+    int lattice = -1, nx = 0, ny = 0, nz = 0;
     cudaStream_t stream = nullptr;
     std::vector<uint8_t> mask;        // empty: no walls
 };
@@ -2089,11 +2073,9 @@ extern "C" int tlb_step_noalloc(const tlb_params *pin, const uint8_t *mask, floa
     int D = Dof(p->lattice);
     float *rho = (float *)base;
     float *phi = (float *)(base + NOALLOC_PHI);
-    int4 *tiles = (int4 *)(base + NOALLOC_TILES);
-    uint8_t *type = base + NOALLOC_FLAGS;
+    uint8_t *type = base + NOALLOC_FLAGS, *wall_tiles = base + NOALLOC_WALLS;
     unsigned *status = (unsigned *)(base + NOALLOC_STATUS);
-    BatchEntry *entries = (BatchEntry *)(base + NOALLOC_ENTRIES);
-    // Node flags (the rules of tlb_set_solid) and the tile table of the
+    // Node flags (the rules of tlb_set_solid) and the wall tiles of the
     // lattice.  The array keeps them from the previous call on this device:
     // when the lattice, the sizes, the mask and the stream are the same, that
     // copy is used again and the host pass over the mask skipped (the kernels
@@ -2106,32 +2088,24 @@ extern "C" int tlb_step_noalloc(const tlb_params *pin, const uint8_t *mask, floa
         std::vector<uint8_t> flags;
         std::vector<int> ghosts;
         node_flags(p->nx, p->ny, p->nz, D, mask, flags, ghosts);
-        int TX = D == 2 ? Launch<2>::tile_dims(0) : Launch<3>::tile_dims(0);
-        int TY = D == 2 ? Launch<2>::tile_dims(1) : Launch<3>::tile_dims(1);
-        int TZ = D == 2 ? Launch<2>::tile_dims(2) : Launch<3>::tile_dims(2);
-        std::vector<int4> tl;
-        for (int z = 0; z < p->nz; z += TZ)
-            for (int y = 0; y < p->ny; y += TY)
-                for (int x = 0; x < p->nx; x += TX) tl.push_back(make_int4(0, x, y, z));
-        if (tl.size() > NOALLOC_M) return fail(TLB_E_INVAL, "tile table exceeds the scratch array");
         CUDA_TRY(cudaMemcpyAsync(type, flags.data(), (size_t)N, cudaMemcpyHostToDevice, st));
-        CUDA_TRY(cudaMemcpyAsync(tiles, tl.data(), tl.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+        if (D == 2) Launch<2>::wall_tiles(dp, type, wall_tiles, st);
+        else Launch<3>::wall_tiles(dp, type, wall_tiles, st);
+        CUDA_TRY(cudaGetLastError());
         nd.lattice = p->lattice;
         nd.nx = p->nx;
         nd.ny = p->ny;
         nd.nz = p->nz;
         nd.stream = st;
-        nd.ntiles = (int)tl.size();
         if (mask) nd.mask.assign(mask, mask + N);
         else nd.mask.clear();
         nd.have_geom = true;
     }
-    // one batch entry per buffer parity: parity 0 reads f, g and writes
-    // f_tmp, g_tmp; parity 1 the other way round (no tensor maps: the step
-    // kernel copies a tile's own populations with cp.async)
-    BatchEntry ent[2];
+    // parity 0 reads f, g and writes f_tmp, g_tmp; parity 1 the other way round
+    // (no tensor maps: the step kernel copies a tile's own populations with
+    // cp.async)
+    BatchEntry ent[2] = {};
     for (int par = 0; par < 2; ++par) {
-        ent[par] = BatchEntry{};
         ent[par].p = dp;
         ent[par].f_in = par ? f_tmp : f;
         ent[par].f_out = par ? f : f_tmp;
@@ -2141,18 +2115,19 @@ extern "C" int tlb_step_noalloc(const tlb_params *pin, const uint8_t *mask, floa
         ent[par].phi = phi;
         ent[par].type = type;
         ent[par].status = status;
-        for (int k = 0; k < 3; ++k) ent[par].tm[k] = nullptr;
+        ent[par].wall_tiles = wall_tiles;
     }
-    CUDA_TRY(cudaMemcpyAsync(entries, ent, sizeof(ent), cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(unsigned), st));
-    const int ntiles = nd.ntiles;
     int cur = 0;
     for (int k = 0; k < nsteps; ++k) {
+        // the step kernel reads the wall tiles ahead of its wait for what
+        // precedes it, so the first launch behind a rebuild starts after it
+        const bool pdl = same || k > 0;
         if (D == 2) {
-            Launch<2>::step_batch(entries + cur, tiles, ntiles, 0, st);
+            Launch<2>::step(ent[cur], st, pdl);
         } else {
-            Launch<3>::moments_batch(entries + cur, tiles, ntiles, 0, st);
-            Launch<3>::step_batch(entries + cur, tiles, ntiles, 0, st);
+            Launch<3>::moments_step(ent[cur], st, pdl);
+            Launch<3>::step(ent[cur], st);
         }
         cur ^= 1;
     }

@@ -129,17 +129,17 @@ struct Bulk {
 // Psi of Eq. PsiEOS and its printed derivative.
 __device__ __forceinline__ Bulk bulk_terms(const DevParams &p, float rho, float phi)
 {
-    float C1 = (rho - p.rho_l) * p.inv_rgl;            // (rho - rho_l)/(rho_g - rho_l)
-    float C2 = 0.5f * (1.0f + phi * p.inv_chi - C1);
-    float C3 = 0.5f * (1.0f - phi * p.inv_chi - C1);
+    const float C1 = (rho - p.rho_l) * p.inv_rgl;            // (rho - rho_l)/(rho_g - rho_l)
+    const float C2 = 0.5f * (fmaf(phi, p.inv_chi, 1.0f) - C1);
+    const float C3 = 0.5f * (fmaf(-phi, p.inv_chi, 1.0f) - C1);
     float br = p.b * rho;
     float psi, dpsi;
     if (p.eos == 0) {
         // Carnahan-Starling, Eq. PsiEOS and its printed derivative
         float q = br - 4.0f;
         float lr = __logf(rho);
-        psi = rho * (p.C - p.a * rho - 8.0f * p.RT * (br - 6.0f) / (q * q) + p.RT * lr);
-        dpsi = p.C - 2.0f * p.a * rho + p.RT * (1.0f + lr) + 16.0f * p.RT * (br - 12.0f) / (q * q * q);
+        psi = rho * fmaf(p.RT, lr, fmaf(-p.a, rho, p.C) - 8.0f * p.RT * (br - 6.0f) / (q * q));
+        dpsi = fmaf(p.RT, 1.0f + lr, fmaf(-2.0f * p.a, rho, p.C)) + 16.0f * p.RT * (br - 12.0f) / (q * q * q);
     } else {
         // van der Waals: Psi = rho (C - a rho + RT ln(rho/(1 - b rho)));
         // Peng-Robinson adds - a A/(2 sqrt2 b) ln((b rho + sqrt2 - 1)/(sqrt2 + 1 - b rho))
@@ -157,12 +157,12 @@ __device__ __forceinline__ Bulk bulk_terms(const DevParams &p, float rho, float 
         }
     }
     float g2 = gpoly(C2), g3 = gpoly(C3);
-    float fb = 0.5f * p.lam1 * (psi - p.Psi0) + 0.5f * p.lam2 * C2 * C2 * (1.0f - C2) * (1.0f - C2) +
-               0.5f * p.lam3 * C3 * C3 * (1.0f - C3) * (1.0f - C3);
+    const float s2 = fmaf(-C2, C2, C2), s3 = fmaf(-C3, C3, C3);
+    float fb = fmaf(p.hl1, psi - p.Psi0, fmaf(0.5f * p.lam2 * s2, s2, 0.5f * p.lam3 * s3 * s3));
     Bulk r;
-    r.murB = 0.5f * p.lam1 * dpsi + (p.lam2 * g2 + p.lam3 * g3) * p.inv_drho;
-    r.mupB = (p.lam2 * g2 - p.lam3 * g3) * p.inv_chi;
-    r.p0 = rho * r.murB + phi * r.mupB - fb;
+    r.murB = fmaf(p.hl1, dpsi, fmaf(p.lam2, g2, p.lam3 * g3) * p.inv_drho);
+    r.mupB = fmaf(p.lam2, g2, -(p.lam3 * g3)) * p.inv_chi;
+    r.p0 = fmaf(rho, r.murB, fmaf(phi, r.mupB, -fb));
     return r;
 }
 
@@ -189,9 +189,9 @@ struct Fac {
 
 __device__ __forceinline__ Fac eq_factors(float u)
 {
-    float s = sqrtf(1.0f + 3.0f * u * u);
+    float s = sqrtf(fmaf(3.0f * u, u, 1.0f));
     float A = 2.0f - s;
-    float B = (2.0f * u + s) / (1.0f - u);
+    float B = fmaf(2.0f, u, s) / (1.0f - u);
     Fac r;
     r.f0 = (2.0f / 3.0f) * A;
     r.fp = (1.0f / 6.0f) * A * B;
@@ -205,8 +205,9 @@ __device__ __forceinline__ float fac_of(const Fac &f, int c) { return c == 0 ? f
 // (series y^2/2 - y^3/6 + ...)
 __device__ __forceinline__ float phi_ent(float y, float l)
 {
-    if (fabsf(y) < 1e-2f) return y * y * (0.5f + y * (-1.0f / 6.0f + y * (1.0f / 12.0f - y * (1.0f / 20.0f))));
-    return (1.0f + y) * l - y;
+    if (fabsf(y) < 1e-2f)
+        return y * y * fmaf(y, fmaf(y, fmaf(y, -1.0f / 20.0f, 1.0f / 12.0f), -1.0f / 6.0f), 0.5f);
+    return fmaf(1.0f + y, l, -y);
 }
 
 // Entropic alpha: the non-trivial root of H(f' + alpha D) = H(f')
@@ -230,30 +231,15 @@ __device__ __forceinline__ float phi_ent(float y, float l)
 // units in the last place of alpha, and moves f by less than 4e-8 of itself)
 // and as the start of Halley's method (third order, from h, h', h''),
 // bracketed by [1, alpha_max), above it (nodes at the interface).
-// FPA: accessor of f'_i.
 constexpr float ALPHA_SERIES_MAX = 0.1f;
-template <int Q, class FPA>
-__device__ __forceinline__ float alpha_series_a(const FPA &fp, const float (&x)[Q])
+__device__ __forceinline__ float alpha_series(float a2, float a3, float a4, float a5, float a6, float a7)
 {
-    float a2 = 0.f, a3 = 0.f, a4 = 0.f, a5 = 0.f, a6 = 0.f, a7 = 0.f;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const float x2 = x[i] * x[i];
-        const float fx2 = fp(i) * x2, fx4 = fx2 * x2;
-        a2 += fx2;
-        a3 += fx2 * x[i];
-        a4 += fx4;
-        a5 += fx4 * x[i];
-        a6 += fx4 * x2;
-        a7 += fx4 * x2 * x[i];
-    }
-    if (!(a2 > 0.f)) return 2.0f;
     const float r = 1.0f / a2;
     const float b3 = a3 * r, b4 = a4 * r, b5 = a5 * r, b6 = a6 * r, b7 = a7 * r;
     const float b33 = b3 * b3;
     const float e1 = b3 * (1.0f / 3.0f);
-    const float e2 = (2.0f / 9.0f) * (2.0f * b33 - 3.0f * b4);
-    const float e3 = (297.0f * b5 - 420.0f * b3 * b4 + 170.0f * b33 * b3) * (1.0f / 270.0f);
+    const float e2 = (2.0f / 9.0f) * fmaf(2.0f, b33, -3.0f * b4);
+    const float e3 = fmaf(297.0f, b5, b3 * fmaf(170.0f, b33, -420.0f * b4)) * (1.0f / 270.0f);
     const float e4 = (1026.0f * b3 * b5 + 540.0f * b4 * b4 - 702.0f * b6 - 1305.0f * b33 * b4 + 380.0f * b33 * b33) *
                      (1.0f / 405.0f);
     const float e5 = (15390.0f * b7 - 23184.0f * b3 * b6 - 24570.0f * b4 * b5 + 30114.0f * b33 * b5 +
@@ -262,16 +248,16 @@ __device__ __forceinline__ float alpha_series_a(const FPA &fp, const float (&x)[
     return 2.0f + e1 + e2 + e3 + e4 + e5;
 }
 
-template <int Q>
-struct RegPop {
-    const float (&v)[Q];
-    __device__ __forceinline__ float operator()(int i) const { return v[i]; }
-};
-
-template <int Q>
-__device__ __forceinline__ float alpha_series(const float (&fp)[Q], const float (&x)[Q])
+// The first two terms alone, from a_2 .. a_4: e3 + e4 + e5 is below
+// (297 + 420 + 170)/270 max|x|^3, which times beta x_i <= max|x| / 2 moves f by
+// less than 1.7 max|x|^4 of itself -- 1.7e-8, less than half a rounding, at
+// ALPHA_SHORT_MAX.
+constexpr float ALPHA_SHORT_MAX = 0.01f;
+__device__ __forceinline__ float alpha_short(float a2, float a3, float a4)
 {
-    return alpha_series_a<Q>(RegPop<Q>{fp}, x);
+    const float r = 1.0f / a2;
+    const float b3 = a3 * r, b4 = a4 * r;
+    return fmaf(2.0f / 9.0f, fmaf(2.0f * b3, b3, -3.0f * b4), fmaf(b3, 1.0f / 3.0f, 2.0f));
 }
 
 // Root of h in (1, alpha_max) from the start al.  h(1) < 0 always; when h is
@@ -281,12 +267,14 @@ __device__ __forceinline__ float alpha_series(const float (&fp)[Q], const float 
 // iteration: the third-order convergence leaves an error of order 1e-9
 // alpha, below the FP32 evaluation noise of h (about 1e-6 alpha at
 // max|x| = 0.5).
-template <int Q, class FPA>
-__device__ __forceinline__ float alpha_newton_a(const FPA &fp, const float (&x)[Q], float amax, float al)
+// L, stride: Q floats of shared memory of the thread's own, which hold ln(1 +
+// x_i) (in registers they would be the third array beside f' and x).
+template <int Q>
+__device__ __forceinline__ float alpha_newton(const float (&fp)[Q], const float (&x)[Q], float amax, float al, float *L,
+                                              int stride)
 {
-    float L[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) L[i] = log1pf(x[i]);
+    for (int i = 0; i < Q; ++i) L[i * stride] = log1pf(x[i]);
     const float bound = amax * (1.0f - 1e-6f);
     float lo = 1.0f, hi = bound;
     bool probed = false;
@@ -300,9 +288,9 @@ __device__ __forceinline__ float alpha_newton_a(const FPA &fp, const float (&x)[
         for (int i = 0; i < Q; ++i) {
             const float y = a * x[i];
             const float ly = log1pf(y);
-            const float f = fp(i);
-            h += f * (phi_ent(y, ly) - y * L[i]);
-            d1 += f * x[i] * (ly - L[i]);
+            const float f = fp[i], l = L[i * stride];
+            h = fmaf(f, fmaf(-y, l, phi_ent(y, ly)), h);
+            d1 = fmaf(f * x[i], ly - l, d1);
             d2 += f * x[i] * x[i] / (1.0f + y);
         }
         if (a == bound) {
@@ -333,12 +321,6 @@ __device__ __forceinline__ float alpha_newton_a(const FPA &fp, const float (&x)[
         a = nxt;
     }
     return a;
-}
-
-template <int Q>
-__device__ __forceinline__ float alpha_newton(const float (&fp)[Q], const float (&x)[Q], float amax, float al)
-{
-    return alpha_newton_a<Q>(RegPop<Q>{fp}, x, amax, al);
 }
 
 // ---------------------------------------------------------------------------

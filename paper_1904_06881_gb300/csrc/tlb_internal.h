@@ -28,6 +28,7 @@ struct DevParams {
     float lam1, lam2, lam3;
     float chi, inv_chi;
     float a, b, RT, C, Psi0;
+    float b4, hl1;       // b/4, lam1/2
     float rho_l, rho_g;
     float inv_drho;      // 1/(rho_l - rho_g)
     float inv_rgl;       // 1/(rho_g - rho_l)
@@ -62,14 +63,17 @@ enum : unsigned {
     STATUS_TIMEOUT = 2u,   // a bounded wait for a tile's tensor copies gave up
 };
 
-// Auxiliary outputs of the step kernel (AUX mode); any may be null.
+// Auxiliary outputs of the field pass (AUX mode); any may be null.
 struct AuxOut {
     float *p0, *mur, *mup, *F[3], *P[6];
 };
 
-enum StepMode { MODE_STEP = 0, MODE_INIT = 1, MODE_AUX = 2 };
+enum FieldMode { MODE_INIT = 1, MODE_AUX = 2 };
 
-// Batched execution: one tile -> lattice table entry.
+constexpr int WALL_WORDS = 32;
+
+// One lattice for the stepping kernels: by value when stepped alone, an entry of
+// a table when batched.
 struct BatchEntry {
     DevParams p;
     float *f_in, *f_out;
@@ -81,7 +85,15 @@ struct BatchEntry {
     // f_in and g_in (FP32 g) or of its FP32 rest channel and FP16 moving
     // channels, for TMA copies of a tile's own populations; null otherwise
     const void *tm[3];
+    const uint8_t *wall_tiles;  // per tile (x fastest): 1 with a solid node in the tile + halo 2
+    // lattices of up to 32 WALL_WORDS tiles stepped alone: the same as bits
+    int wall_known;
+    uint32_t wall_bits[WALL_WORDS];
 };
+
+// lattices whose node offsets in bytes pass 32 bits (D2Q9: 155 GB and more of
+// populations; in D3Q27 they would be 464 GB)
+inline bool big_lattice(long long N) { return N >= (1LL << 30); }
 
 // Launchers implemented per lattice (D = 2: tlb_d2q9.cu, D = 3: tlb_d3q27.cu).
 template <int D>
@@ -89,8 +101,8 @@ struct Launch {
     static int Q();
     static void moments(const DevParams &p, const DevState &s, cudaStream_t st);
     static void ghosts(const DevParams &p, const DevState &s, cudaStream_t st);
-    static void step(const DevParams &p, const DevState &s, int mode, const float *u_init, AuxOut aux,
-                     cudaStream_t st);
+    static void field_pass(const DevParams &p, const DevState &s, int mode, const float *u_init, AuxOut aux,
+                           cudaStream_t st);
     static void fields(const DevParams &p, const DevState &s, float *u_out, cudaStream_t st);
     static void diagnostics(const DevParams &p, const DevState &s, double *partials, int nblocks, double *out,
                             cudaStream_t st);
@@ -104,8 +116,15 @@ struct Launch {
     static void moments_batch(const BatchEntry *entries, const int4 *tiles, int ntiles, int g_fp16, cudaStream_t st);
     // variant: D2Q9 register budget, 0 = 3 CTAs/SM (80 registers), 1 = 4 CTAs/SM
     // (64 registers), -1 = 4 CTAs/SM beyond one wave of 3 CTAs/SM; D3Q27 has one
-    static void step_batch(const BatchEntry *entries, const int4 *tiles, int ntiles, int g_fp16, cudaStream_t st,
-                           int variant = -1);
+    // big: one of the lattices is a big_lattice
+    static void step_batch(const BatchEntry *entries, const int4 *tiles, int ntiles, int g_fp16, bool big,
+                           cudaStream_t st, int variant = -1);
+    // one lattice alone (the same step): `pdl` false where the launch must not
+    // start before what precedes it on the stream has completed
+    static void moments_step(const BatchEntry &e, cudaStream_t st, bool pdl = true);
+    static void step(const BatchEntry &e, cudaStream_t st, bool pdl = true);
+    static void wall_tiles(const DevParams &p, const uint8_t *type, uint8_t *out, cudaStream_t st);
+    static int tiles(const DevParams &p);
     static int tile_dims(int a);
 };
 
