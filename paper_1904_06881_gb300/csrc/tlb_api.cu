@@ -454,19 +454,8 @@ struct tlb_ctx {
     uint8_t *wall_tiles = nullptr;    // per tile: 1 with a solid node within two links
     uint32_t wall_bits[WALL_WORDS] = {};   // the same as bits (lattices of few tiles)
     int wall_known = 0;
-    // one CUDA graph per buffer parity holding the launches of a step (D3Q27)
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-    cudaStream_t cap_stream = nullptr;
+    int backwards = 0;                // D3Q27: f and g larger than the L2 cache
 };
-
-static void drop_graphs(tlb_ctx *c)
-{
-    for (int k = 0; k < 2; ++k)
-        if (c->gexec[k]) {
-            cudaGraphExecDestroy(c->gexec[k]);
-            c->gexec[k] = nullptr;
-        }
-}
 
 static int Qof(int lattice) { return lattice == TLB_D3Q27 ? 27 : 9; }
 
@@ -601,6 +590,7 @@ static BatchEntry make_entry(const tlb_ctx *c, int cur)
     e.status = c->s.status;
     for (int k = 0; k < 3; ++k) e.tm[k] = c->tmaps ? (const void *)(c->tmaps + 3 * cur + k) : nullptr;
     e.wall_tiles = c->wall_tiles;
+    e.backwards = c->backwards;
     e.wall_known = c->wall_known;
     std::memcpy(e.wall_bits, c->wall_bits, sizeof(e.wall_bits));
     return e;
@@ -767,6 +757,10 @@ extern "C" int tlb_create_ex(const tlb_params *pin, tlb_ctx **out)
         ALLOC_LATE(c->wall_tiles, nt);
         cudaMemsetAsync(c->wall_tiles, 0, nt, c->stream);
         c->wall_known = nt <= 32 * WALL_WORDS;         // no walls yet
+        int dev = 0, l2 = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+        c->backwards = c->D == 3 && Q * N * 4 + gb > (size_t)l2;
     }
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
@@ -805,8 +799,6 @@ extern "C" void tlb_destroy(tlb_ctx *c)
 {
     if (!c) return;
     cudaStreamSynchronize(c->stream);
-    drop_graphs(c);
-    if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     dev_free_all(c->owned);
     delete c;
 }
@@ -893,7 +885,6 @@ extern "C" int tlb_set_solid(tlb_ctx *c, const uint8_t *mask)
     std::vector<uint8_t> t;
     node_flags(c->p.nx, c->p.ny, c->p.nz, c->D, mask, t, c->ghost_host);
     c->type_host = t;
-    drop_graphs(c);
     CUDA_TRY(cudaMemcpyAsync(c->s.type, t.data(), N, cudaMemcpyHostToDevice, c->stream));
     size_t ng = c->ghost_host.size();
     if (ng > c->ghosts_cap) {
@@ -1029,26 +1020,6 @@ static void issue_step_on(tlb_ctx *c, cudaStream_t st)
     issue_phase(c, 2, st);
 }
 
-// Capture the launches of a step for the current buffer parity.
-static int capture_step(tlb_ctx *c)
-{
-    int par = c->s.cur;
-    if (c->gexec[par]) return TLB_OK;
-    if (!c->cap_stream) CUDA_TRY(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
-    cudaGraph_t g = nullptr;
-    CUDA_TRY(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-    issue_step_on(c, c->cap_stream);
-    cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
-    if (e != cudaSuccess) return fail(TLB_E_CUDA, "step capture: %s", cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&c->gexec[par], g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-        c->gexec[par] = nullptr;
-        return fail(TLB_E_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
-    }
-    return TLB_OK;
-}
-
 extern "C" int tlb_step(tlb_ctx *c, int nsteps)
 {
     NvtxRange range("tlb_step");
@@ -1056,14 +1027,10 @@ extern "C" int tlb_step(tlb_ctx *c, int nsteps)
     if (nsteps < 0) return fail(TLB_E_INVAL, "nsteps < 0");
     const int per = launches_per_step(c->D);
     for (int k = 0; k < nsteps; ++k) {
-        if (per == 1) {
-            // a single launch: direct (a one-node graph costs more to launch)
-            issue_step_on(c, c->stream);
-        } else {
-            int rc = capture_step(c);
-            if (rc) return rc;
-            CUDA_TRY(cudaGraphLaunch(c->gexec[c->s.cur], c->stream));
-        }
+        // launched directly: each kernel's start overlaps its predecessor's end
+        // (programmatic dependent launch), which a graph per step stops at every
+        // step (D3Q27 32 x 32 x 20: 26 -> 24.6 us a step, 101 x 100 x 100: 2 %)
+        issue_step_on(c, c->stream);
         c->s.cur ^= 1;
         c->steps += 1;
         c->launches += per;
