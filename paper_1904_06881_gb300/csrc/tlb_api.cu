@@ -824,58 +824,79 @@ extern "C" int tlb_set_stream(tlb_ctx *c, void *stream)
     return TLB_OK;
 }
 
+// out[n] = OR of in over the node and its neighbours along one axis of a
+// periodic lattice: `len` nodes `stride` apart in each of the lattice's lines
+// (stride 1: along x)
+static void spread(const uint8_t *in, uint8_t *out, size_t N, size_t len, size_t stride)
+{
+    const size_t block = len * stride;
+    for (size_t b = 0; b < N; b += block)
+        for (size_t k = 0; k < len; ++k) {
+            const uint8_t *c = in + b + k * stride;
+            const uint8_t *m = in + b + (k ? k - 1 : len - 1) * stride, *p = in + b + (k + 1 < len ? k + 1 : 0) * stride;
+            uint8_t *o = out + b + k * stride;
+            for (size_t x = 0; x < stride; ++x) o[x] = c[x] | m[x] | p[x];
+        }
+}
+
+// the same over the 3^D nodes around a node (in is overwritten)
+static void spread_all(std::vector<uint8_t> &in, std::vector<uint8_t> &tmp, int nx, int ny, int nz, int D)
+{
+    const size_t N = in.size(), row = (size_t)nx;
+    for (size_t b = 0; b < N; b += row) {
+        const uint8_t *c = in.data() + b;
+        uint8_t *o = tmp.data() + b;
+        o[0] = c[row - 1] | c[0] | c[1];
+        for (size_t x = 1; x + 1 < row; ++x) o[x] = c[x - 1] | c[x] | c[x + 1];
+        o[row - 1] = c[row - 2] | c[row - 1] | c[0];
+    }
+    spread(tmp.data(), in.data(), N, (size_t)ny, row);
+    if (D == 3) {
+        in.swap(tmp);
+        spread(tmp.data(), in.data(), N, (size_t)nz, row * (size_t)ny);
+    }
+}
+
 // Node flags and ghost list of a periodic lattice from its solid mask (NULL:
 // no walls): solid, ghost (solid with a fluid lattice neighbour), first layer
 // (fluid with a solid lattice neighbour), wall axes, and NEAR (fluid off the
 // first layer with a first-layer neighbour: where the wetting force acts).
+// Neighbourhoods of 3^D nodes are taken one axis after another, on bytes along
+// the memory order (64^3 nodes: 20 ms when every node looked its 26 neighbours
+// up, which a server paid for each request it admitted).
 static void node_flags(int nx, int ny, int nz, int D, const uint8_t *mask, std::vector<uint8_t> &t,
                        std::vector<int> &ghosts)
 {
-    auto at = [&](int x, int y, int z) -> long long {
-        x = ((x % nx) + nx) % nx;
-        y = ((y % ny) + ny) % ny;
-        z = ((z % nz) + nz) % nz;
-        return (long long)x + (long long)nx * ((long long)y + (long long)ny * z);
-    };
-    auto solid = [&](long long n) { return mask != nullptr && mask[n] != 0; };
-    long long N = (long long)nx * ny * nz;
-    t.assign((size_t)N, 0);
+    const size_t N = (size_t)nx * ny * nz, row = (size_t)nx, plane = row * (size_t)ny;
+    t.assign(N, 0);
     ghosts.clear();
-    const int zr = D == 3 ? 1 : 0;
-    for (int z = 0; z < nz; ++z)
-        for (int y = 0; y < ny; ++y)
-            for (int x = 0; x < nx; ++x) {
-                long long n = at(x, y, z);
-                bool s = solid(n), touch = false;
-                for (int dz = -zr; dz <= zr; ++dz)
-                    for (int dy = -1; dy <= 1; ++dy)
-                        for (int dx = -1; dx <= 1; ++dx)
-                            if ((dx || dy || dz) && solid(at(x + dx, y + dy, z + dz)) != s) touch = true;
-                uint8_t v = s ? TLB_SOLID : 0;
-                if (s && touch) {
-                    v |= TLB_GHOST;
-                    ghosts.push_back((int)n);
-                }
-                if (!s) {
-                    if (touch) v |= TLB_FIRST;
-                    if (solid(at(x + 1, y, z)) || solid(at(x - 1, y, z))) v |= TLB_WALLX;
-                    if (solid(at(x, y + 1, z)) || solid(at(x, y - 1, z))) v |= TLB_WALLY;
-                    if (D == 3 && (solid(at(x, y, z + 1)) || solid(at(x, y, z - 1)))) v |= TLB_WALLZ;
-                }
-                t[n] = v;
+    if (!mask) return;
+    std::vector<uint8_t> solid(N), s(N), f(N), tmp(N);
+    for (size_t n = 0; n < N; ++n) {
+        solid[n] = mask[n] != 0;
+        s[n] = solid[n];
+        f[n] = !solid[n];
+    }
+    spread_all(s, tmp, nx, ny, nz, D);            // a solid node around
+    spread_all(f, tmp, nx, ny, nz, D);            // a fluid node around
+    for (size_t n = 0; n < N; ++n)
+        t[n] = solid[n] ? (f[n] ? TLB_SOLID | TLB_GHOST : TLB_SOLID) : (s[n] ? TLB_FIRST : 0);
+    // wall axes, on first-layer nodes alone (no other has a solid neighbour)
+    for (size_t z = 0, n = 0; z < (size_t)nz; ++z)
+        for (size_t y = 0; y < (size_t)ny; ++y)
+            for (size_t x = 0; x < row; ++x, ++n) {
+                if (t[n] & TLB_GHOST) ghosts.push_back((int)n);
+                if (!(t[n] & TLB_FIRST)) continue;
+                const size_t xo = n - x, yo = n - y * row, zo = n - z * plane;
+                if (solid[xo + (x + 1 < row ? x + 1 : 0)] | solid[xo + (x ? x - 1 : row - 1)]) t[n] |= TLB_WALLX;
+                if (solid[yo + (y + 1 < (size_t)ny ? y + 1 : 0) * row] | solid[yo + (y ? y - 1 : (size_t)ny - 1) * row]) t[n] |= TLB_WALLY;
+                if (D == 3 && (solid[zo + (z + 1 < (size_t)nz ? z + 1 : 0) * plane] | solid[zo + (z ? z - 1 : (size_t)nz - 1) * plane]))
+                    t[n] |= TLB_WALLZ;
             }
-    for (int z = 0; z < nz; ++z)
-        for (int y = 0; y < ny; ++y)
-            for (int x = 0; x < nx; ++x) {
-                long long n = at(x, y, z);
-                if (t[n] & (TLB_SOLID | TLB_FIRST)) continue;
-                bool near = false;
-                for (int dz = -zr; dz <= zr; ++dz)
-                    for (int dy = -1; dy <= 1; ++dy)
-                        for (int dx = -1; dx <= 1; ++dx)
-                            if ((dx || dy || dz) && (t[at(x + dx, y + dy, z + dz)] & TLB_FIRST)) near = true;
-                if (near) t[n] |= TLB_NEAR;
-            }
+    for (size_t n = 0; n < N; ++n) f[n] = (t[n] & TLB_FIRST) != 0;
+    spread_all(f, tmp, nx, ny, nz, D);            // a first-layer node around
+    for (size_t n = 0; n < N; ++n)
+        if (f[n] && !(t[n] & (TLB_SOLID | TLB_FIRST))) t[n] |= TLB_NEAR;
 }
 
 extern "C" int tlb_set_solid(tlb_ctx *c, const uint8_t *mask)
