@@ -298,7 +298,7 @@ def run_ours(args):
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": cfg,
         "roofline": roofline(Q, N, kern_ms, peak, peak_kind,
-                             "step_batch_kernel<D3Q27> (ghost layer, stencils, force, collision, stream)",
+                             "step_kernel<D3Q27> (ghost layer, stencils, force, collision, stream)",
                              wl["name"]),
         "whole_step": {"bytes_per_node": algorithmic_bytes(Q, 1) + 8 * Q + 9,
                        "note": "moments pass (read f, g, flag; write rho, phi) + step kernel",
@@ -352,7 +352,7 @@ def run_ours(args):
                "gpu_launches": int(la1), "clocks": clk1.summary(), "angles_deg": [30, 60, 120],
                "l2": "256 MB buffer written before every timed step; steps timed alone",
                "roofline": roofline(l1.Q, l1.N, kms1, peak, peak_kind,
-                                    "step_batch_kernel<D2Q9> (moments, ghost layer, stencils, force, collision, "
+                                    "step_kernel<D2Q9> (moments, ghost layer, stencils, force, collision, "
                                     "stream)", c1["name"])})
     result["c1_capillary"] = d1
     l1.close()
@@ -368,7 +368,7 @@ def run_ours(args):
             result["big_lattices"].append({
                 "workload": bw["name"], "value": round(world * bl.N / (bms * 1e-3) / 1e6, 2), "unit": "MLUPS",
                 "ms_per_step": round(bms, 4), "gpu_launches": int(blaunch), "l2": "state larger than L2; no flush",
-                "roofline": roofline(bl.Q, bl.N, bkms, peak, peak_kind, "step_batch_kernel", bw["name"])})
+                "roofline": roofline(bl.Q, bl.N, bkms, peak, peak_kind, "step_kernel", bw["name"])})
             bl.close()
     if rank == 0 and not args.no_batch:
         result["batched"] = batched_sweep()

@@ -22,15 +22,6 @@
 
 namespace tlb {
 
-template <class T>
-struct CharOf {
-    using type = char;
-};
-template <class T>
-struct CharOf<const T> {
-    using type = const char;
-};
-
 // ---- packed FP32 pairs ----
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -47,18 +38,6 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b)
         " sub.rn.ftz.f32x2 c, a, b;\n mov.b64 {%0, %1}, c;\n}\n"
         : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return r;
-}
-
-// Element idx of an array: a 32-bit byte offset on the array's base, which the
-// hardware adds in the access (one integer instruction less for each of a
-// node's 36 or 54 loads and stores: D2Q9 2048 x 2048 192 -> 177 us a step).
-// BIG: lattices of 2^30 nodes and more, whose offsets need 64 bits.
-template <bool BIG, class T>
-__device__ __forceinline__ T *elem(T *base, int idx)
-{
-    if (BIG) return base + (long long)idx;
-    using C = typename CharOf<T>::type;
-    return reinterpret_cast<T *>(reinterpret_cast<C *>(base) + (unsigned)idx * (unsigned)sizeof(T));
 }
 
 // weight class of the pair k: 0 faces, 1 edges, 2 corners
@@ -256,15 +235,21 @@ struct StepShared {
     static constexpr int RX = TX + 4, RY = TY + 4, RZ = D == 3 ? TZ + 4 : 1;
     static constexpr int SX = TX + 2, SY = TY + 2, SZ = D == 3 ? TZ + 2 : 1;
     static constexpr int NR = RX * RY * RZ, NS = SX * SY * SZ;
+    // row length of rp.  D3Q27: 34 = SX mod 16, so that a half-warp of the tensor
+    // stage that crosses a row's end meets no bank twice (1.4 % of the 192 x 192 x
+    // 128 step).  With the staged populations a CTA stays below the 100 KB beyond
+    // which the L1 cache shrinks (staging rows of 16-byte pieces, where tensor
+    // copies are not possible, passed it and was 5 to 8 % slower).
+    static constexpr int PX = D == 3 ? 34 : RX;
     // D2Q9 tiles with ghost nodes: flags and moments of the tile + halo 2
     // widened by EM nodes, the reach of the ghost layer (for theta in
     // [20, 160] deg a ghost node's samples lie at most 3 nodes along the wall
     // and 1 across from it; farther nodes are read from global memory)
     static constexpr int EM = 3, BX = RX + 2 * EM, BY = RY + 2 * EM, NB = D == 2 ? BX * BY : 1;
     float4 qa[NS];                        // Q of the tile + halo 1: D3Q27 {xx, yy, zz, xy}; D2Q9 {xx, yy, xy, mu_phi}
-    float2 rp[NR];                        // rho, phi of the tile + halo 2
+    float2 rp[PX * RY * RZ];              // rho, phi of the tile + halo 2
     float2 qb[D == 3 ? NS : 1];           // D3Q27 {xz, yz}
-    float mu[D == 3 ? NS : 1];            // D3Q27 mu_phi
+    float mu[D == 3 ? NT : 1];            // D3Q27 mu_phi of the tile's nodes
     float2 box[NB];
     short glist[D == 2 ? NR : 1];         // the region's ghost slots, one per thread in the ghost pass
     uint8_t type[NS];                     // node flags of the tile + halo 1
@@ -470,7 +455,7 @@ __device__ __forceinline__ void own_copies_3d(const BatchEntry &e, int x0, int y
     const int tid = threadIdx.x;
             if (use_tma) {
                 // one thread: a box of TX x TY x TZ nodes x all directions per array
-                // (x0 is a multiple of 8 nodes: 16-byte aligned inner coordinate)
+                // (x0 is a multiple of 16 nodes: 16-byte aligned inner coordinate)
                 if (tid == 0) {
                     mbar_init(&sh.tma_bar, 1);
                     const unsigned bytes = (unsigned)(Q * NT * 4) +
@@ -553,7 +538,8 @@ __device__ __forceinline__ void gather_3d(const BatchEntry &e, int x0, int y0, i
             for (int j = 0; j < PER; ++j) {
                 const int k = tid + NT * j;
                 if (k < NP)
-                    reinterpret_cast<float4 *>(sh.rp)[k] = make_float4(lr[j].x, lp[j].x, lr[j].y, lp[j].y);
+                    reinterpret_cast<float4 *>(sh.rp)[(k / RH) * (S::PX / 2) + k % RH] =
+                        make_float4(lr[j].x, lp[j].x, lr[j].y, lp[j].y);
             }
             __syncthreads();
             return;
@@ -579,7 +565,7 @@ __device__ __forceinline__ void gather_3d(const BatchEntry &e, int x0, int y0, i
     for (int j = 0; j < PER; ++j) {
         const int k = tid + NT * j;
         if (k >= NR) break;
-        sh.rp[k] = make_float2(lr[j], lp[j]);
+        sh.rp[(k / RX) * S::PX + k % RX] = make_float2(lr[j], lp[j]);
         if (WALLS) {
             sh.rtype[k] = lt[j];
             ghost |= (lt[j] & TLB_GHOST) != 0;
@@ -592,7 +578,7 @@ __device__ __forceinline__ void gather_3d(const BatchEntry &e, int x0, int y0, i
             if (!(sh.rtype[k] & TLB_GHOST)) continue;      // unfilled slots hold TLB_SOLID alone
             float gr, gp;
             ghost_value<3>(p, acc, x0 - 2 + k % RX, y0 - 2 + (k / RX) % RY, z0 - 2 + k / (RX * RY), gr, gp);
-            sh.rp[k] = make_float2(gr, gp);
+            sh.rp[(k / RX) * S::PX + k % RX] = make_float2(gr, gp);
         }
     }
     __syncthreads();
@@ -686,14 +672,17 @@ __device__ __forceinline__ void tensor_stage(const DevParams &p, int x0, int y0,
             for (int j = 0; j < (D == 2 ? 3 : 6); ++j) q[j] = 0.f;
             mup = 0.f;
         } else {
-            node_q<D, RX, RY>(p, sh.rp + c, q, mup);
+            node_q<D, S::PX, RY>(p, sh.rp + (lx + 1) + S::PX * ((ly + 1) + RY * (lz + HZ)), q, mup);
         }
         if constexpr (D == 2) {
             sh.qa[k] = make_float4(q[0], q[1], q[2], mup);
         } else {
             sh.qa[k] = make_float4(q[0], q[1], q[2], q[3]);
             sh.qb[k] = make_float2(q[4], q[5]);
-            sh.mu[k] = mup;
+            // for the tile's own nodes
+            const int tx = lx - 1, ty = ly - 1, tz = lz - 1;
+            if ((unsigned)tx < (unsigned)S::TX && (unsigned)ty < (unsigned)S::TY && (unsigned)tz < (unsigned)S::TZ)
+                sh.mu[tx + S::TX * (ty + S::TY * tz)] = mup;
         }
     }
 }
@@ -754,7 +743,7 @@ __device__ __forceinline__ float node_force(const DevParams &p, const StepShared
         wall_force<D>(qc, sh.type, tc, sc, F);
     }
     if (WALLS) wetting_force<D>(p, sh.type, tc, sc, r, ph, F);
-    return D == 2 ? sh.qa[sc].w : sh.mu[sc];
+    return D == 2 ? sh.qa[sc].w : sh.mu[threadIdx.x];
 }
 
 // Where a node's populations go: push streaming with halfway bounce-back.
@@ -1055,7 +1044,7 @@ __device__ __forceinline__ void step_tile(const BatchEntry &e, int x0, int y0, i
     const int sc = (tx + 1) + SX * ((ty + 1) + SY * (tz + HZ));
     const uint8_t tc = WALLS ? sh.type[sc] : (uint8_t)0;
     if (tc & TLB_SOLID) return;
-    const float2 rph = sh.rp[(tx + 2) + RX * ((ty + 2) + RY * (tz + 2 * HZ))];
+    const float2 rph = sh.rp[(tx + 2) + S::PX * ((ty + 2) + RY * (tz + 2 * HZ))];
     const float r = rph.x, ph = rph.y;
     float F[D];
     const float mup = node_force<D, WALLS>(p, sh, sc, tc, r, ph, F);
