@@ -8,18 +8,18 @@
 //        moving populations as half[Q-1][N] scaled by 16
 //   rho, phi : float[N] moments of the current state, written by the moments
 //              kernel (ghost values are computed in shared memory by the step
-//              kernels; only the auxiliary-output and allocation-free paths
-//              write them to these arrays)
+//              kernels; only the passes over initial and auxiliary fields write
+//              them to these arrays)
 //   type : uint8[N]  node flags (TLB_SOLID, TLB_FIRST, TLB_GHOST, TLB_NEAR, wall axes)
-// One step, through a tile -> lattice table (the same kernels for one lattice
-// and for a batch):
-//   D2Q9  : step_batch_kernel alone -- rho, phi of the tile + halo 2 summed
-//           from the populations, ghost layer, stencils, chemical potentials,
+// One step (one lattice: step_kernel, moments_step_kernel; a batch: the same tile
+// code through a tile -> lattice table, step_batch_kernel, moments_batch_kernel):
+//   D2Q9  : the step kernel alone -- rho, phi of the tile + halo 2 summed from
+//           the populations, ghost layer, stencils, chemical potentials,
 //           pressure tensor (halo 1), force with wall rules, ELBM collision of
 //           f (entropic alpha), LBGK of g, push streaming with halfway
 //           bounce-back;
-//   D3Q27 : moments_batch_kernel (rho = 1 + sum_i f~_i, phi = sum_i g_i), then
-//           step_batch_kernel as above with rho, phi read from the moments.
+//   D3Q27 : the moments pass (rho = 1 + sum_i f~_i, phi = sum_i g_i), then the
+//           step kernel as above with rho, phi read from the moments.
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
