@@ -1024,9 +1024,12 @@ static int launches_per_step(int D) { return D == 2 ? 1 : 2; }
 // The launches of one step of a lattice alone (the tile code of the batched
 // kernels, so alone and batched results are bit-identical).  Phase 0 is the
 // moments pass (D3Q27 only), phase 2 the step kernel.
-static void issue_phase(tlb_ctx *c, int phase, cudaStream_t st)
+// `recorded`: the launch may run later, when tlb_set_solid has changed the walls,
+// so it takes the tiles' wall flags from memory and not the entry's copy of them.
+static void issue_phase(tlb_ctx *c, int phase, cudaStream_t st, bool recorded)
 {
-    const BatchEntry e = make_entry(c, c->s.cur);
+    BatchEntry e = make_entry(c, c->s.cur);
+    if (recorded) e.wall_known = 0;
     if (c->D == 2) {
         if (phase == 2) Launch<2>::step(e, st);
     } else {
@@ -1035,10 +1038,20 @@ static void issue_phase(tlb_ctx *c, int phase, cudaStream_t st)
     }
 }
 
-static void issue_step_on(tlb_ctx *c, cudaStream_t st)
+static void issue_step_on(tlb_ctx *c, cudaStream_t st, bool recorded)
 {
-    issue_phase(c, 0, st);
-    issue_phase(c, 2, st);
+    issue_phase(c, 0, st, recorded);
+    issue_phase(c, 2, st, recorded);
+}
+
+// whether launches on the stream are being recorded into a graph (or cannot be
+// told, as on the default stream beside such a recording)
+static bool is_recording(cudaStream_t st)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();                   // the launches report what is wrong
+    return true;
 }
 
 extern "C" int tlb_step(tlb_ctx *c, int nsteps)
@@ -1047,11 +1060,12 @@ extern "C" int tlb_step(tlb_ctx *c, int nsteps)
     if (!c) return fail(TLB_E_INVAL, "null context");
     if (nsteps < 0) return fail(TLB_E_INVAL, "nsteps < 0");
     const int per = launches_per_step(c->D);
+    const bool recorded = is_recording(c->stream);
     for (int k = 0; k < nsteps; ++k) {
         // launched directly: each kernel's start overlaps its predecessor's end
         // (programmatic dependent launch), which a graph per step stops at every
         // step (D3Q27 32 x 32 x 20: 26 -> 24.6 us a step, 101 x 100 x 100: 2 %)
-        issue_step_on(c, c->stream);
+        issue_step_on(c, c->stream, recorded);
         c->s.cur ^= 1;
         c->steps += 1;
         c->launches += per;
@@ -1067,7 +1081,7 @@ extern "C" int tlb_step_phase(tlb_ctx *c, int phase)
     if (phase < 0 || phase > 2) return fail(TLB_E_INVAL, "phase must be 0, 1 or 2");
     if (phase == 1) return TLB_OK;        // the ghost layer is filled inside phase 2
     if (phase == 0 && c->D == 2) return TLB_OK;   // D2Q9 step kernels sum their moments
-    issue_phase(c, phase, c->stream);
+    issue_phase(c, phase, c->stream, is_recording(c->stream));
     if (phase == 2) {
         c->s.cur ^= 1;
         c->steps += 1;

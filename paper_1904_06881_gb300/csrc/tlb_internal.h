@@ -92,7 +92,8 @@ struct BatchEntry {
     // with FP16 g); where they fit, the order buys nothing and put the tiles of a
     // drop on the wall last (75 x 61 x 47: 12 % slower).
     int backwards;
-    // lattices of up to 32 WALL_WORDS tiles stepped alone: the same as bits
+    // lattices of up to 32 WALL_WORDS tiles stepped alone and at once: the same as
+    // bits (0 in a recorded launch, which may run after the walls have changed)
     int wall_known;
     uint32_t wall_bits[WALL_WORDS];
 };

@@ -1,0 +1,83 @@
+"""tlb_step recorded into a CUDA graph on the caller's stream: the replayed
+steps take the solid mask that is set when they run, not the one of the
+recording."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_1904_06881_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _wl(lattice, mask_kind):
+    nx, ny, nz = (96, 40, 1) if lattice == W.D2Q9 else (32, 16, 12)
+    z, y, x = np.mgrid[0:nz, 0:ny, 0:nx].astype(np.float64)
+    d2 = (x - 0.45 * nx) ** 2 + (y - 0.5 * ny) ** 2 + (0.0 if nz == 1 else (z - 0.5 * nz) ** 2)
+    C2 = 0.5 * (1.0 - np.tanh((np.sqrt(d2) - 5.0) / 2.0))
+    rho, phi = W.phase_fields(C2, np.zeros_like(C2))
+    mask = np.zeros((nz, ny, nx), np.uint8)
+    if mask_kind == "block":
+        mask[: min(nz, 5), 3:9, nx - 9:nx - 4] = 1
+    return dict(name="capture", lattice=lattice, nx=nx, ny=ny, nz=nz, mask=mask, rho=rho, phi=phi,
+                params=W.base_params(wetting=W.WET_FORCE, kw_rho=0.05))
+
+
+class _Driver:
+    """The driver's stream capture, for a stream given as an integer handle."""
+
+    def __init__(self):
+        self.cu = ctypes.CDLL("libcuda.so.1")
+
+    def begin(self, stream):
+        assert self.cu.cuStreamBeginCapture_v2(ctypes.c_void_p(stream), 1) == 0        # this thread's calls only
+
+    def end(self, stream):
+        graph = ctypes.c_void_p()
+        return self.cu.cuStreamEndCapture(ctypes.c_void_p(stream), ctypes.byref(graph)), graph
+
+    def instantiate(self, graph):
+        ex = ctypes.c_void_p()
+        assert self.cu.cuGraphInstantiateWithFlags(ctypes.byref(ex), graph, ctypes.c_ulonglong(0)) == 0
+        return ex
+
+    def launch(self, ex, stream):
+        assert self.cu.cuGraphLaunch(ex, ctypes.c_void_p(stream)) == 0
+
+    def destroy(self, graph, ex):
+        self.cu.cuGraphExecDestroy(ex)
+        self.cu.cuGraphDestroy(graph)
+
+
+@pytest.mark.parametrize("lattice", [W.D2Q9, W.D3Q27])
+def test_recorded_steps_follow_a_new_mask(lattice):
+    import torch
+
+    from paper_1904_06881_gb300 import tlb
+
+    drv = _Driver()
+    open_, block = _wl(lattice, "none"), _wl(lattice, "block")
+    s = torch.cuda.Stream()
+    lat = tlb.lattice_from_workload(open_)
+    lat.step(2)
+    lat.sync()
+    tlb.tlb_set_stream(lat.h, s.cuda_stream)
+    drv.begin(s.cuda_stream)
+    tlb.tlb_step(lat.h, 4)                     # an even number: the buffers' roles return
+    rc, graph = drv.end(s.cuda_stream)
+    assert rc == 0
+    ex = drv.instantiate(graph)
+    for wl in (block, open_, block):
+        lat.set_solid(wl["mask"])
+        lat.init_fields(wl["rho"], wl["phi"])
+        drv.launch(ex, s.cuda_stream)
+        torch.cuda.synchronize()
+        ref = tlb.lattice_from_workload(wl)
+        ref.step(4)
+        fl = wl["mask"].reshape(-1) == 0
+        for a, b in zip(lat.populations(), ref.populations()):
+            assert np.array_equal(a[:, fl], b[:, fl])
+        ref.close()
+    drv.destroy(graph, ex)
+    lat.close()
