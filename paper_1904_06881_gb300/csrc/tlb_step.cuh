@@ -69,7 +69,9 @@ __device__ __forceinline__ float eos_pressure(const DevParams &p, float rho)
         return rho * fmaf(p.RT * num, r * r * r, -(p.a * rho));
     }
     const float br = p.b * rho;
-    const float rep = p.RT / (1.0f - br);
+    // no state beyond the pole at b rho = 1, where Psi has no logarithm either: not a
+    // number, which the collision reports
+    const float rep = br < 1.0f ? p.RT / (1.0f - br) : __int_as_float(0x7fffffff);
     if (p.eos == 1) return rho * fmaf(-p.a, rho, rep);                      // van der Waals
     return rho * (rep - p.aA * rho / fmaf(br, 2.0f - br, 1.0f));            // Peng-Robinson
 }
