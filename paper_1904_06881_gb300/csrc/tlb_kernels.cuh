@@ -394,7 +394,8 @@ __global__ void __launch_bounds__(256) field_kernel(DevParams p, float *__restri
     __shared__ float sQ[NC][NS];          // Q = rho c_s^2 I - P of the tile + halo 1
     __shared__ float smu[NS];
     __shared__ uint8_t stype[NS], srt[NR];
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * Tile<D>::Z;
+    int x0, y0, z0;
+    tile_origin<D>(p, blockIdx.x, x0, y0, z0);
     const int tid = threadIdx.x;
     // rho, phi and flags of the tile + halo 2, all of a thread's slots loaded
     // in one round, then the ghost layer of Sec. IV
@@ -664,9 +665,8 @@ template <int D>
 void Launch<D>::field_pass(const DevParams &p, const DevState &s, int mode, const float *u_init, AuxOut aux,
                            cudaStream_t st)
 {
-    const dim3 grid((p.nx + Tile<D>::X - 1) / Tile<D>::X, (p.ny + Tile<D>::Y - 1) / Tile<D>::Y,
-                    (p.nz + Tile<D>::Z - 1) / Tile<D>::Z);
-    const dim3 block(Tile<D>::X * Tile<D>::Y * Tile<D>::Z);
+    // one dimension: the others end at 65535, which a lattice of many tile rows passes
+    const int grid = tiles(p), block = Tile<D>::X * Tile<D>::Y * Tile<D>::Z;
     float *f = s.f[s.cur];
     void *g = s.g[s.cur];
     if (mode == MODE_AUX)
