@@ -335,9 +335,9 @@ __device__ __forceinline__ void gather_2d(const BatchEntry &e, int x0, int y0, S
     auto load = [&](int s) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            fa[s][i] = __ldg(elem<BIG>(e.f_in + (long long)i * p.N, na[s]));
+            fa[s][i] = *elem<BIG>(e.f_in + (long long)i * p.N, na[s]);
             if (sizeof(GT) == 4 || i == 0) {
-                ga[s][i] = __ldg(elem<BIG>((const float *)e.g_in + (long long)i * p.N, na[s]));
+                ga[s][i] = *elem<BIG>((const float *)e.g_in + (long long)i * p.N, na[s]);
             } else {
                 // the value GIO<__half>::ld returns, from one load of the raw half
                 gh[s][i] = *elem<BIG>((const __half *)((const char *)e.g_in + 4 * p.N) + (long long)(i - 1) * p.N, na[s]);
@@ -535,8 +535,8 @@ __device__ __forceinline__ void gather_3d(const BatchEntry &e, int x0, int y0, i
                                       : (int)chk_node(x0 - 2 + 2 * (k - RH * row) +
                                                           p.nx * (y0 - 2 + row % RY + p.ny * (z0 - 2 + row / RY)), p);
                 if (k < NP) {
-                    lr[j] = __ldg(reinterpret_cast<const float2 *>(e.rho + n));
-                    lp[j] = __ldg(reinterpret_cast<const float2 *>(e.phi + n));
+                    lr[j] = *reinterpret_cast<const float2 *>(e.rho + n);
+                    lp[j] = *reinterpret_cast<const float2 *>(e.phi + n);
                 }
             }
             own_copies();
@@ -563,8 +563,8 @@ __device__ __forceinline__ void gather_3d(const BatchEntry &e, int x0, int y0, i
         const bool in = k < NR && X < p.nx + 2 && Y < p.ny + 2 && Z < p.nz + 2;
         const int n = in ? node_near(p, X, Y, Z) : 0;
         if (WALLS) lt[j] = in ? __ldg(e.type + n) : (uint8_t)TLB_SOLID;
-        lr[j] = in ? __ldg(e.rho + n) : 0.f;
-        lp[j] = in ? __ldg(e.phi + n) : 0.f;
+        lr[j] = in ? e.rho[n] : 0.f;
+        lp[j] = in ? e.phi[n] : 0.f;
     }
     own_copies();
 #pragma unroll
