@@ -15,6 +15,7 @@
 #include <deque>
 #include <map>
 #include <mutex>
+#include <new>
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -902,12 +903,17 @@ static void node_flags(int nx, int ny, int nz, int D, const uint8_t *mask, std::
 extern "C" int tlb_set_solid(tlb_ctx *c, const uint8_t *mask)
 {
     if (!c || !mask) return fail(TLB_E_INVAL, "null argument");
-    long long N = c->N;
+    const size_t N = (size_t)c->N;
+    // all that can run out of memory comes first: a call that fails for it leaves
+    // the context with the mask it had
     std::vector<uint8_t> t;
-    node_flags(c->p.nx, c->p.ny, c->p.nz, c->D, mask, t, c->ghost_host);
-    c->type_host = t;
-    CUDA_TRY(cudaMemcpyAsync(c->s.type, t.data(), N, cudaMemcpyHostToDevice, c->stream));
-    size_t ng = c->ghost_host.size();
+    std::vector<int> ghosts;
+    try {
+        node_flags(c->p.nx, c->p.ny, c->p.nz, c->D, mask, t, ghosts);
+    } catch (const std::bad_alloc &) {
+        return fail(TLB_E_NOMEM, "no host memory for the node flags of %zu nodes", N);
+    }
+    const size_t ng = ghosts.size();
     if (ng > c->ghosts_cap) {
         void *ptr;
         int rc = dev_alloc(c->owned, &ptr, ng * sizeof(int), &c->bytes);
@@ -915,6 +921,9 @@ extern "C" int tlb_set_solid(tlb_ctx *c, const uint8_t *mask)
         c->ghosts_dev = (int *)ptr;
         c->ghosts_cap = ng;
     }
+    c->type_host.swap(t);
+    c->ghost_host.swap(ghosts);
+    CUDA_TRY(cudaMemcpyAsync(c->s.type, c->type_host.data(), N, cudaMemcpyHostToDevice, c->stream));
     if (ng) CUDA_TRY(cudaMemcpyAsync(c->ghosts_dev, c->ghost_host.data(), ng * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     DISPATCH(c, wall_tiles(c->dp, c->s.type, c->wall_tiles, c->stream));
     CUDA_TRY(cudaGetLastError());
