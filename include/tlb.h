@@ -95,7 +95,9 @@ int tlb_version(int *major, int *minor, int *sm);
 
 /* Device allocator used for every later allocation (NULL restores
  * cudaMalloc/cudaFree).  alloc(bytes, user) returns device memory or NULL;
- * free_(ptr, user) releases it. */
+ * free_(ptr, user) releases it.  Memory on 64-byte boundaries gives the D3Q27
+ * kernels their widest copies; batches want 16 (else TLB_E_INVAL), contexts 4
+ * (8 for blocks of doubles, the sums of tlb_diagnostics). */
 int tlb_set_allocator(void *(*alloc)(size_t bytes, void *user), void (*free_)(void *ptr, void *user),
                       void *user);
 

@@ -576,6 +576,12 @@ static bool encode_tensor_maps(const tlb_ctx *c, CUtensorMap maps[6])
     return true;
 }
 
+// whether every row of rho and phi starts on an 8-byte boundary
+static int rows_paired(const DevParams &p, const float *rho, const float *phi)
+{
+    return (p.nx & 1) == 0 && (((uintptr_t)rho | (uintptr_t)phi) & 7) == 0;
+}
+
 // the lattice as the stepping kernels take it, reading population buffer `cur`
 static BatchEntry make_entry(const tlb_ctx *c, int cur)
 {
@@ -592,6 +598,7 @@ static BatchEntry make_entry(const tlb_ctx *c, int cur)
     for (int k = 0; k < 3; ++k) e.tm[k] = c->tmaps ? (const void *)(c->tmaps + 3 * cur + k) : nullptr;
     e.wall_tiles = c->wall_tiles;
     e.backwards = c->backwards;
+    e.paired = rows_paired(c->dp, c->s.rho, c->s.phi);
     e.wall_known = c->wall_known;
     std::memcpy(e.wall_bits, c->wall_bits, sizeof(e.wall_bits));
     return e;
@@ -1313,6 +1320,15 @@ static bool any_big(const std::vector<tlb_ctx *> &ctxs)
     return false;
 }
 
+// a batch's tables are read in words of their entries' alignment
+static int tables_aligned(BatchEntry *const entries[2], const int4 *tiles)
+{
+    if (((uintptr_t)tiles & (alignof(int4) - 1)) == 0 &&
+        (((uintptr_t)entries[0] | (uintptr_t)entries[1]) & (alignof(BatchEntry) - 1)) == 0)
+        return TLB_OK;
+    return fail(TLB_E_INVAL, "the allocator's memory is not aligned to 16 bytes");
+}
+
 static int build_plan(tlb_ctx *const *ctxs, int n, BatchPlan &plan, cudaStream_t st)
 {
     int D = ctxs[0]->D;
@@ -1340,6 +1356,7 @@ static int build_plan(tlb_ctx *const *ctxs, int n, BatchPlan &plan, cudaStream_t
     plan.entries[1] = (BatchEntry *)ptr;
     if ((rc = dev_alloc(plan.owned, &ptr, tiles.size() * sizeof(int4), nullptr))) return rc;
     plan.tiles = (int4 *)ptr;
+    if ((rc = tables_aligned(plan.entries, plan.tiles))) return rc;
     CUDA_TRY(cudaMemcpyAsync(plan.entries[0], e0.data(), n * sizeof(BatchEntry), cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMemcpyAsync(plan.entries[1], e1.data(), n * sizeof(BatchEntry), cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMemcpyAsync(plan.tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
@@ -1543,6 +1560,7 @@ extern "C" int tlb_batch_create(tlb_ctx *const *ctxs, int n, const tlb_batch_con
         b->entries[par] = (BatchEntry *)ptr;
     }
     if (rc == 0 && (rc = dev_alloc(b->owned, &ptr, ntiles * sizeof(int4), nullptr)) == 0) b->tiles = (int4 *)ptr;
+    if (rc == 0) rc = tables_aligned(b->entries, b->tiles);
     if (rc == 0) rc = batch_write_entries(b);
     if (rc == 0) rc = batch_write_tiles(b);
     if (rc == 0 && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
@@ -2127,6 +2145,7 @@ extern "C" int tlb_step_noalloc(const tlb_params *pin, const uint8_t *mask, floa
         ent[par].type = type;
         ent[par].status = status;
         ent[par].wall_tiles = wall_tiles;
+        ent[par].paired = rows_paired(dp, rho, phi);
     }
     CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(unsigned), st));
     int cur = 0;

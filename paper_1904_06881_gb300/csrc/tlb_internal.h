@@ -92,6 +92,9 @@ struct BatchEntry {
     // with FP16 g); where they fit, the order buys nothing and put the tiles of a
     // drop on the wall last (75 x 61 x 47: 12 % slower).
     int backwards;
+    // D3Q27: the rows of rho and phi start on 8-byte boundaries (two nodes a load);
+    // nx even, and what a caller's allocator gave
+    int paired;
     // lattices of up to 32 WALL_WORDS tiles stepped alone and at once: the same as
     // bits (0 in a recorded launch, which may run after the walls have changed)
     int wall_known;

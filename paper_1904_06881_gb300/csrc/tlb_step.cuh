@@ -524,7 +524,7 @@ __device__ __forceinline__ void gather_3d(const BatchEntry &e, int x0, int y0, i
         // the region of a tile away from the lattice's edges lies in memory as
         // rows of RX nodes: two nodes a load where the rows are 8-byte aligned
         if (x0 >= 2 && y0 >= 2 && z0 >= 2 && x0 + TX + 2 <= p.nx && y0 + TY + 2 <= p.ny &&
-            z0 + S::TZ + 2 <= p.nz && (p.nx & 1) == 0) {
+            z0 + S::TZ + 2 <= p.nz && e.paired) {
             constexpr int RH = RX / 2, NP = RH * RY * RZ, PER = (NP + NT - 1) / NT;
             float2 lr[PER], lp[PER];
 #pragma unroll
