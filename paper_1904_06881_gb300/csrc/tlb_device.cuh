@@ -253,7 +253,7 @@ __device__ __forceinline__ float phi_ent(float y, float l)
 // and as the start of Halley's method (third order, from h, h', h''),
 // bracketed by [1, alpha_max), above it (nodes at the interface).
 constexpr float ALPHA_SERIES_MAX = 0.1f;
-__device__ __forceinline__ float alpha_series(float a2, float a3, float a4, float a5, float a6, float a7)
+__host__ __device__ __forceinline__ float alpha_series(float a2, float a3, float a4, float a5, float a6, float a7)
 {
     const float r = 1.0f / a2;
     const float b3 = a3 * r, b4 = a4 * r, b5 = a5 * r, b6 = a6 * r, b7 = a7 * r;
@@ -269,16 +269,20 @@ __device__ __forceinline__ float alpha_series(float a2, float a3, float a4, floa
     return 2.0f + e1 + e2 + e3 + e4 + e5;
 }
 
-// The first two terms alone, from a_2 .. a_4: e3 + e4 + e5 is below
-// (297 + 420 + 170)/270 max|x|^3, which times beta x_i <= max|x| / 2 moves f by
-// less than 1.7 max|x|^4 of itself -- 1.7e-8, less than half a rounding, at
-// ALPHA_SHORT_MAX.
-constexpr float ALPHA_SHORT_MAX = 0.01f;
-__device__ __forceinline__ float alpha_short(float a2, float a3, float a4)
+// The first two terms alone, from a_2 .. a_4.  |b_k| <= max|x|^(k - 2), so e3 is
+// below (297 + 420 + 170)/270 max|x|^3 and e4 below 9.8 max|x|^4: together below
+// 3.3e-9 at ALPHA_SHORT_MAX, a thirtieth of what rounding alpha = 2 + ... leaves
+// (half a unit in its last place, 1.2e-7 above 2 and 6e-8 below).  In FP32 the
+// root is then as far from the exact one as with all five terms (1.19e-7 at most,
+// 5.4e-8 on average); at 0.01 it was 3.4e-7 and 1.5e-7.  Steps with the limit at
+// 0.01, here, and without the short form: D2Q9 2048 x 2048 171.0, 171.2, 180.0 us,
+// D3Q27 192 x 192 x 128 746, 764, 764.
+constexpr float ALPHA_SHORT_MAX = 0.001f;
+__host__ __device__ __forceinline__ float alpha_short(float a2, float a3, float a4)
 {
     const float r = 1.0f / a2;
     const float b3 = a3 * r, b4 = a4 * r;
-    return fmaf(2.0f / 9.0f, fmaf(2.0f * b3, b3, -3.0f * b4), fmaf(b3, 1.0f / 3.0f, 2.0f));
+    return 2.0f + fmaf(b3, 1.0f / 3.0f, (2.0f / 9.0f) * fmaf(2.0f * b3, b3, -3.0f * b4));
 }
 
 // Root of h in (1, alpha_max) from the start al.  h(1) < 0 always; when h is

@@ -854,9 +854,8 @@ __device__ __forceinline__ void collide_f(const BatchEntry &e, float r, float ph
         }
     }
     // Entropic alpha (Eq. EntropyEquation) from x_i = D_i / f'_i.  The moments
-    // a_2 .. a_4 of x alone give alpha = 2 + e1 + e2, which moves f by less
-    // than (5/3) max|x|^4 of itself: 1.7e-8, below half a rounding, at the
-    // bound ALPHA_SHORT_MAX = 0.01.  Above it the moments a_5 .. a_7 complete
+    // a_2 .. a_4 of x alone give alpha = 2 + e1 + e2, to a fraction of its
+    // rounding up to max|x| = ALPHA_SHORT_MAX.  Above it the moments a_5 .. a_7 complete
     // the fifth-order series, above ALPHA_SERIES_MAX Halley's method follows.
     float al = 2.0f, fmn, xmax, a2, a3, a4;
     {
