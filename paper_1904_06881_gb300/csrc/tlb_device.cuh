@@ -190,14 +190,14 @@ __device__ __forceinline__ Bulk bulk_terms(const DevParams &p, float rho, float 
 // ELBM beta of a node: the fluid's beta, or with per-component viscosities
 // the beta of the concentration-weighted mean viscosity (concentrations
 // clipped to [0, 1]), nu = (1/beta - 1)/6.
-__device__ __forceinline__ float local_beta(const DevParams &p, float rho, float phi)
+__host__ __device__ __forceinline__ float local_beta(const DevParams &p, float rho, float phi)
 {
     if (!p.nu_on) return p.beta;
     const float C1 = (rho - p.rho_l) * p.inv_rgl;
-    const float C2 = 0.5f * (1.0f + phi * p.inv_chi - C1), C3 = 0.5f * (1.0f - phi * p.inv_chi - C1);
+    const float C2 = 0.5f * (fmaf(phi, p.inv_chi, 1.0f) - C1), C3 = 0.5f * (fmaf(-phi, p.inv_chi, 1.0f) - C1);
     const float c1 = fminf(fmaxf(C1, 0.f), 1.f), c2 = fminf(fmaxf(C2, 0.f), 1.f), c3 = fminf(fmaxf(C3, 0.f), 1.f);
-    const float nu = (c1 * p.nu[0] + c2 * p.nu[1] + c3 * p.nu[2]) / (c1 + c2 + c3);
-    return 1.0f / (6.0f * nu + 1.0f);
+    const float nu = fmaf(c1, p.nu[0], fmaf(c2, p.nu[1], c3 * p.nu[2])) / (c1 + c2 + c3);
+    return 1.0f / fmaf(6.0f, nu, 1.0f);
 }
 
 // ---------------------------------------------------------------------------
@@ -258,15 +258,16 @@ __host__ __device__ __forceinline__ float alpha_series(float a2, float a3, float
     const float r = 1.0f / a2;
     const float b3 = a3 * r, b4 = a4 * r, b5 = a5 * r, b6 = a6 * r, b7 = a7 * r;
     const float b33 = b3 * b3;
-    const float e1 = b3 * (1.0f / 3.0f);
-    const float e2 = (2.0f / 9.0f) * fmaf(2.0f, b33, -3.0f * b4);
-    const float e3 = fmaf(297.0f, b5, b3 * fmaf(170.0f, b33, -420.0f * b4)) * (1.0f / 270.0f);
-    const float e4 = (1026.0f * b3 * b5 + 540.0f * b4 * b4 - 702.0f * b6 - 1305.0f * b33 * b4 + 380.0f * b33 * b33) *
-                     (1.0f / 405.0f);
-    const float e5 = (15390.0f * b7 - 23184.0f * b3 * b6 - 24570.0f * b4 * b5 + 30114.0f * b33 * b5 +
-                      31080.0f * b3 * b4 * b4 - 36295.0f * b33 * b3 * b4 + 8260.0f * b33 * b33 * b3) *
-                     (1.0f / 5670.0f);
-    return 2.0f + e1 + e2 + e3 + e4 + e5;
+    // e5 first: the smallest terms, and the last use of the highest moments
+    const float e5 = fmaf(b3, fmaf(b33, fmaf(8260.0f, b33, -36295.0f * b4), fmaf(31080.0f * b4, b4, -23184.0f * b6)),
+                          fmaf(b5, fmaf(30114.0f, b33, -24570.0f * b4), 15390.0f * b7));
+    const float e4 = fmaf(b33, fmaf(380.0f, b33, -1305.0f * b4), fmaf(1026.0f * b3, b5, fmaf(540.0f * b4, b4, -702.0f * b6)));
+    const float e3 = fmaf(297.0f, b5, b3 * fmaf(170.0f, b33, -420.0f * b4));
+    const float e2 = fmaf(2.0f, b33, -3.0f * b4);
+    float s = fmaf(e4, 1.0f / 405.0f, e5 * (1.0f / 5670.0f));
+    s = fmaf(e3, 1.0f / 270.0f, s);
+    s = fmaf(e2, 2.0f / 9.0f, s);
+    return 2.0f + fmaf(b3, 1.0f / 3.0f, s);
 }
 
 // The first two terms alone, from a_2 .. a_4.  |b_k| <= max|x|^(k - 2), so e3 is
@@ -329,7 +330,7 @@ __device__ __forceinline__ float alpha_newton(const float (&fp)[Q], const float 
         float nxt;
         if (d1 > 0.f) {
             const float s = h / d1;
-            const float step = s / (1.0f - 0.5f * s * d2 / d1);   // Halley's update
+            const float step = s / fmaf(-0.5f * s, d2 / d1, 1.0f);   // Halley's update
             if (fabsf(step) <= 1e-3f * al) return fminf(al - step, bound);
             nxt = al - step;
             if (!(nxt > lo && nxt < hi)) {
@@ -371,8 +372,9 @@ struct NodesGlobal {
 
 // The ghost value of one fluid-facing axis direction: (yx, yy, yz) is the
 // first fluid node along `axis`, m1 its moments; `acc` a node accessor.
+#pragma nv_exec_check_disable
 template <int D, class A>
-__device__ void ghost_axis(const DevParams &p, const A &acc, int yx, int yy, int yz, int axis, float2 m1, float &gr,
+__host__ __device__ void ghost_axis(const DevParams &p, const A &acc, int yx, int yy, int yz, int axis, float2 m1, float &gr,
                            float &gp)
 {
     // Coordinates are kept in scalars (an array indexed by the run-time axis
@@ -403,8 +405,8 @@ __device__ void ghost_axis(const DevParams &p, const A &acc, int yx, int yy, int
     float dr0, dp0, dr1 = 0.f, dp1 = 0.f;
     diff(ux, uy, uz, dr0, dp0);
     if (D == 3) diff(vx, vy, vz, dr1, dp1);
-    const float nr = sqrtf(dr0 * dr0 + dr1 * dr1), npp = sqrtf(dp0 * dp0 + dp1 * dp1);
-    const float dot = dr0 * dp0 + dr1 * dp1;
+    const float nr = sqrtf(fmaf(dr0, dr0, dr1 * dr1)), npp = sqrtf(fmaf(dp0, dp0, dp1 * dp1));
+    const float dot = fmaf(dr0, dp0, dr1 * dp1);
     // interface identification (Sec. IV.B): 0 = 1-2, 1 = 1-3, 2 = 2-3
     int pair;
     if (nr < 0.01f * (p.rho_l - p.rho_g) * p.inv_chi * npp) pair = 2;
@@ -419,10 +421,10 @@ __device__ void ghost_axis(const DevParams &p, const A &acc, int yx, int yy, int
     const float tx = dc0 / nc, ty = D == 3 ? dc1 / nc : 0.f;
     if (p.wetting == TLB_WET_GEOM_EXTRAP) {
         // Eqs. geomamgle, geomding; the second field follows the same interface
-        const float sr = dr0 * tx + (D == 3 ? dr1 * ty : 0.f);
-        const float sp = dp0 * tx + (D == 3 ? dp1 * ty : 0.f);
-        gr = r1 + cot * sr;
-        gp = p1 + cot * sp;
+        const float sr = D == 3 ? fmaf(dr0, tx, dr1 * ty) : dr0 * tx;
+        const float sp = D == 3 ? fmaf(dp0, tx, dp1 * ty) : dp0 * tx;
+        gr = fmaf(cot, sr, r1);
+        gp = fmaf(cot, sp, p1);
         return;
     }
     // geometric interpolation: sample at cot(theta) t_hat in the first fluid layer
@@ -443,12 +445,12 @@ __device__ void ghost_axis(const DevParams &p, const A &acc, int yx, int yy, int
         samp(l0, 0, v0r, v0p);
         samp(l1, 0, v1r, v1p);
         const float t = l - (float)l0;           // linear interpolation on [l0, l1] (Eq. interp2D)
-        gr = v0r + t * (v1r - v0r);
-        gp = v0p + t * (v1p - v0p);
+        gr = fmaf(t, v1r - v0r, v0r);
+        gp = fmaf(t, v1p - v0p, v0p);
         return;
     }
     const float lx = cot * tx, ly = cot * ty;
-    if (sqrtf(lx * lx + ly * ly) < 1e-12f) { gr = r1; gp = p1; return; }
+    if (sqrtf(fmaf(lx, lx, ly * ly)) < 1e-12f) { gr = r1; gp = p1; return; }
     const int X0 = (int)floorf(lx), Y0 = (int)floorf(ly);
     // of the four corners k = 0..3 at (X0 + (k & 1), Y0 + (k >> 1)) of the unit
     // cell around (lx, ly), drop the one nearest to the origin (first of
@@ -469,11 +471,11 @@ __device__ void ghost_axis(const DevParams &p, const A &acc, int yx, int yy, int
     samp(cxx, cyy, v2r, v2p);
     // barycentric coordinates of (lx, ly) in the triangle
     const float e1x = (float)(bx - ax), e1y = (float)(by - ay), e2x = (float)(cxx - ax), e2y = (float)(cyy - ay);
-    const float det = e1x * e2y - e2x * e1y;
+    const float det = fmaf(e1x, e2y, -(e2x * e1y));
     const float px = lx - (float)ax, py = ly - (float)ay;
-    const float b1 = (px * e2y - e2x * py) / det, b2 = (e1x * py - px * e1y) / det;
-    gr = v0r + b1 * (v1r - v0r) + b2 * (v2r - v0r);
-    gp = v0p + b1 * (v1p - v0p) + b2 * (v2p - v0p);
+    const float b1 = fmaf(px, e2y, -(e2x * py)) / det, b2 = fmaf(e1x, py, -(px * e1y)) / det;
+    gr = fmaf(b2, v2r - v0r, fmaf(b1, v1r - v0r, v0r));
+    gp = fmaf(b2, v2p - v0p, fmaf(b1, v1p - v0p, v0p));
 }
 
 }  // namespace tlb
