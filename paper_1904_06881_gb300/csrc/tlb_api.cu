@@ -1042,22 +1042,24 @@ static int launches_per_step(int D) { return D == 2 ? 1 : 2; }
 // moments pass (D3Q27 only), phase 2 the step kernel.
 // `recorded`: the launch may run later, when tlb_set_solid has changed the walls,
 // so it takes the tiles' wall flags from memory and not the entry's copy of them.
-static void issue_phase(tlb_ctx *c, int phase, cudaStream_t st, bool recorded)
+static cudaError_t issue_phase(tlb_ctx *c, int phase, cudaStream_t st, bool recorded)
 {
     BatchEntry e = make_entry(c, c->s.cur);
     if (recorded) e.wall_known = 0;
-    if (c->D == 2) {
-        if (phase == 2) Launch<2>::step(e, st);
-    } else {
-        if (phase == 0) Launch<3>::moments_step(e, st);
-        else if (phase == 2) Launch<3>::step(e, st);
-    }
+    if (c->D == 2) return phase == 2 ? Launch<2>::step(e, st) : cudaSuccess;
+    return phase == 0 ? Launch<3>::moments_step(e, st) : phase == 2 ? Launch<3>::step(e, st) : cudaSuccess;
 }
 
-static void issue_step_on(tlb_ctx *c, cudaStream_t st, bool recorded)
+static cudaError_t issue_step_on(tlb_ctx *c, cudaStream_t st, bool recorded)
 {
-    issue_phase(c, 0, st, recorded);
-    issue_phase(c, 2, st, recorded);
+    const cudaError_t e = issue_phase(c, 0, st, recorded);
+    return e != cudaSuccess ? e : issue_phase(c, 2, st, recorded);
+}
+
+static int fail_launch(cudaError_t e)
+{
+    cudaGetLastError();
+    return fail(TLB_E_CUDA, "step launch: %s", cudaGetErrorString(e));
 }
 
 // whether launches on the stream are being recorded into a graph (or cannot be
@@ -1080,8 +1082,10 @@ extern "C" int tlb_step(tlb_ctx *c, int nsteps)
     for (int k = 0; k < nsteps; ++k) {
         // launched directly: each kernel's start overlaps its predecessor's end
         // (programmatic dependent launch), which a graph per step stops at every
-        // step (D3Q27 32 x 32 x 20: 26 -> 24.6 us a step, 101 x 100 x 100: 2 %)
-        issue_step_on(c, c->stream, recorded);
+        // step (D3Q27 32 x 32 x 20: 26 -> 24.6 us a step, 101 x 100 x 100: 2 %).  A
+        // step that cannot be launched does not count: its buffers keep their roles
+        const cudaError_t e = issue_step_on(c, c->stream, recorded);
+        if (e != cudaSuccess) return fail_launch(e);
         c->s.cur ^= 1;
         c->steps += 1;
         c->launches += per;
@@ -1097,7 +1101,8 @@ extern "C" int tlb_step_phase(tlb_ctx *c, int phase)
     if (phase < 0 || phase > 2) return fail(TLB_E_INVAL, "phase must be 0, 1 or 2");
     if (phase == 1) return TLB_OK;        // the ghost layer is filled inside phase 2
     if (phase == 0 && c->D == 2) return TLB_OK;   // D2Q9 step kernels sum their moments
-    issue_phase(c, phase, c->stream, is_recording(c->stream));
+    const cudaError_t e = issue_phase(c, phase, c->stream, is_recording(c->stream));
+    if (e != cudaSuccess) return fail_launch(e);
     if (phase == 2) {
         c->s.cur ^= 1;
         c->steps += 1;

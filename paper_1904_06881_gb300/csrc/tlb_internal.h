@@ -131,8 +131,8 @@ struct Launch {
                            cudaStream_t st, int variant = -1);
     // one lattice alone (the same step): `pdl` false where the launch must not
     // start before what precedes it on the stream has completed
-    static void moments_step(const BatchEntry &e, cudaStream_t st, bool pdl = true);
-    static void step(const BatchEntry &e, cudaStream_t st, bool pdl = true);
+    static cudaError_t moments_step(const BatchEntry &e, cudaStream_t st, bool pdl = true);
+    static cudaError_t step(const BatchEntry &e, cudaStream_t st, bool pdl = true);
     static void wall_tiles(const DevParams &p, const uint8_t *type, uint8_t *out, cudaStream_t st);
     static int tiles(const DevParams &p);
     static int tile_dims(int a);

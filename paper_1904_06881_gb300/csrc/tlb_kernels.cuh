@@ -713,7 +713,7 @@ void Launch<D>::convert_pop(const DevParams &p, const DevState &s, int dir, doub
 // launch with programmatic stream serialization (the kernel's griddepcontrol.wait
 // orders it after its predecessor's memory operations)
 template <typename... KArgs, typename... Args>
-static void launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, bool pdl,
+static cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, bool pdl,
                        const Args &...args)
 {
     cudaLaunchConfig_t cfg = {};
@@ -726,7 +726,7 @@ static void launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t sme
     attr[0].val.programmaticStreamSerializationAllowed = pdl;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, args...);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 template <int D>
@@ -821,33 +821,33 @@ void Launch<D>::wall_tiles(const DevParams &p, const uint8_t *type, uint8_t *out
 }
 
 template <int D>
-void Launch<D>::moments_step(const BatchEntry &e, cudaStream_t st, bool pdl)
+cudaError_t Launch<D>::moments_step(const BatchEntry &e, cudaStream_t st, bool pdl)
 {
     const int grid = (int)((e.p.N + 255) / 256);
-    if (e.p.g_fp16) launch_pdl(moments_step_kernel<D, __half>, grid, 256, 0, st, pdl, e);
-    else launch_pdl(moments_step_kernel<D, float>, grid, 256, 0, st, pdl, e);
+    if (e.p.g_fp16) return launch_pdl(moments_step_kernel<D, __half>, grid, 256, 0, st, pdl, e);
+    return launch_pdl(moments_step_kernel<D, float>, grid, 256, 0, st, pdl, e);
 }
 
 template <int D, typename GT>
-static void launch_step(const BatchEntry &e, cudaStream_t st, bool pdl)
+static cudaError_t launch_step(const BatchEntry &e, cudaStream_t st, bool pdl)
 {
     constexpr size_t bytes = stage_bytes<D, GT>();
     constexpr int nt = Tile<D>::X * Tile<D>::Y * Tile<D>::Z;
     const int nsm = step_setup<D, GT>(), ntiles = Launch<D>::tiles(e.p);
     if constexpr (D == 2) {
-        if (big_lattice(e.p.N)) launch_pdl(step_kernel<D, GT, 4, true>, ntiles, nt, bytes, st, pdl, e);
-        else if (ntiles > 3 * nsm) launch_pdl(step_kernel<D, GT, 4, false>, ntiles, nt, bytes, st, pdl, e);
-        else launch_pdl(step_kernel<D, GT, 3, false>, ntiles, nt, bytes, st, pdl, e);
+        if (big_lattice(e.p.N)) return launch_pdl(step_kernel<D, GT, 4, true>, ntiles, nt, bytes, st, pdl, e);
+        if (ntiles > 3 * nsm) return launch_pdl(step_kernel<D, GT, 4, false>, ntiles, nt, bytes, st, pdl, e);
+        return launch_pdl(step_kernel<D, GT, 3, false>, ntiles, nt, bytes, st, pdl, e);
     } else {
-        launch_pdl(step_kernel<D, GT, 2, false>, ntiles, nt, bytes, st, pdl, e);
+        return launch_pdl(step_kernel<D, GT, 2, false>, ntiles, nt, bytes, st, pdl, e);
     }
 }
 
 template <int D>
-void Launch<D>::step(const BatchEntry &e, cudaStream_t st, bool pdl)
+cudaError_t Launch<D>::step(const BatchEntry &e, cudaStream_t st, bool pdl)
 {
-    if (e.p.g_fp16) launch_step<D, __half>(e, st, pdl);
-    else launch_step<D, float>(e, st, pdl);
+    if (e.p.g_fp16) return launch_step<D, __half>(e, st, pdl);
+    return launch_step<D, float>(e, st, pdl);
 }
 
 }  // namespace tlb

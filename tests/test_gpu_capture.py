@@ -1,6 +1,7 @@
-"""tlb_step recorded into a CUDA graph on the caller's stream: the replayed
-steps take the solid mask that is set when they run, not the one of the
-recording."""
+"""tlb_step on a stream that is recorded into a CUDA graph: the replayed steps
+take the solid mask that is set when they run, not the one of the recording,
+and a recording that has been invalidated refuses steps, which then do not
+count."""
 import ctypes
 
 import numpy as np
@@ -81,3 +82,34 @@ def test_recorded_steps_follow_a_new_mask(lattice):
         ref.close()
     drv.destroy(graph, ex)
     lat.close()
+
+
+@pytest.mark.parametrize("lattice", [W.D2Q9, W.D3Q27])
+@pytest.mark.parametrize("phases", [False, True])
+def test_steps_that_cannot_be_launched_do_not_count(lattice, phases):
+    import torch
+
+    from paper_1904_06881_gb300 import tlb
+
+    drv, wl, s = _Driver(), _wl(lattice, "block"), torch.cuda.Stream()
+    lat, ref = tlb.lattice_from_workload(wl), tlb.lattice_from_workload(wl)
+    for l in (lat, ref):
+        l.step(3)
+        l.sync()
+    tlb.tlb_set_stream(lat.h, s.cuda_stream)
+    drv.begin(s.cuda_stream)
+    assert tlb.lib().tlb_sync(lat.h) == -3     # a synchronisation, which ends the recording
+    for _ in range(3):                         # an odd number of steps refused
+        rc = tlb.lib().tlb_step_phase(lat.h, 2) if phases else tlb.lib().tlb_step(lat.h, 1)
+        assert rc == -3
+    assert drv.end(s.cuda_stream)[0] != 0
+    assert lat.steps_done == 3
+    for l in (lat, ref):
+        l.step(4)
+        l.sync()
+    assert lat.steps_done == 7
+    fl = wl["mask"].reshape(-1) == 0
+    for a, b in zip(lat.populations(), ref.populations()):
+        assert np.array_equal(a[:, fl], b[:, fl])
+    lat.close()
+    ref.close()
