@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace tlb {
 
 // node flags (uint8 per node)
@@ -104,6 +106,19 @@ struct BatchEntry {
 // lattices whose node offsets in bytes pass 32 bits (D2Q9: 155 GB and more of
 // populations; in D3Q27 they would be 464 GB)
 inline bool big_lattice(long long N) { return N >= (1LL << 30); }
+
+// A positive number that a device is asked for once, per device and not per
+// process: what `ask` sets up (a kernel's shared-memory limit, say) holds on the
+// device it was asked on alone.  Two threads may both ask; 0, a failure, is not
+// kept, nor is the answer of a device beyond the array.
+template <int MAX, class Ask>
+int once_per_device(std::atomic<int> (&known)[MAX], int dev, Ask &&ask)
+{
+    if (dev < 0 || dev >= MAX) return ask();
+    int n = known[dev].load(std::memory_order_acquire);
+    if (n == 0 && (n = ask()) > 0) known[dev].store(n, std::memory_order_release);
+    return n;
+}
 
 // Launchers implemented per lattice (D = 2: tlb_d2q9.cu, D = 3: tlb_d3q27.cu).
 template <int D>

@@ -751,16 +751,20 @@ void Launch<D>::moments_batch(const BatchEntry *entries, const int4 *tiles, int 
     else launch_pdl(moments_batch_kernel<D, float>, ntiles, nt, 0, st, true, entries, tiles);
 }
 
-// per kernel, once per process on the first launch (thread-safe static
-// initialisation): the dynamic shared-memory opt-ins, and the SM count of the
-// device that runs the library (D2Q9: the one-wave bound)
+// per kernel, once per device on the first launch there: the dynamic
+// shared-memory opt-ins; returns the device's SM count (D2Q9: the one-wave bound),
+// 0 if an opt-in failed, whose launch then fails
 template <int D, typename GT>
 static int step_setup()
 {
-    static const int nsm = [] {
+    static std::atomic<int> known[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return once_per_device(known, dev, [dev] {
         constexpr int b = stage_bytes<D, GT>();
-        const auto opt = [](auto *kernel) {
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+        bool ok = true;
+        const auto opt = [&ok](auto *kernel) {
+            ok &= cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b) == cudaSuccess;
         };
         if constexpr (D == 2) {
             opt(step_batch_kernel<D, GT, 3, false>);
@@ -773,12 +777,10 @@ static int step_setup()
             opt(step_batch_kernel<D, GT, 2, false>);
             opt(step_kernel<D, GT, 2, false>);
         }
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
+        int n = 0;
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        return n;
-    }();
-    return nsm;
+        return ok ? n : 0;
+    });
 }
 
 template <int D, typename GT>
