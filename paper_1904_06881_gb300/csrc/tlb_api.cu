@@ -1316,14 +1316,8 @@ struct BatchPlan {
     BatchEntry *entries[2] = {nullptr, nullptr};   // parity of the step
     int4 *tiles = nullptr;
     int ntiles = 0;
+    bool big = false;                              // one of the lattices is a big_lattice
 };
-
-static bool any_big(const std::vector<tlb_ctx *> &ctxs)
-{
-    for (const tlb_ctx *c : ctxs)
-        if (big_lattice(c->N)) return true;
-    return false;
-}
 
 // a batch's tables are read in words of their entries' alignment
 static int tables_aligned(BatchEntry *const entries[2], const int4 *tiles)
@@ -1344,6 +1338,7 @@ static int build_plan(tlb_ctx *const *ctxs, int n, BatchPlan &plan, cudaStream_t
     int TZ = D == 2 ? Launch<2>::tile_dims(2) : Launch<3>::tile_dims(2);
     for (int k = 0; k < n; ++k) {
         tlb_ctx *c = ctxs[k];
+        plan.big |= big_lattice(c->N);
         if (c->D != D) return fail(TLB_E_INVAL, "batched lattices must share the lattice type");
         if (c->p.g_fp16 != ctxs[0]->p.g_fp16) return fail(TLB_E_INVAL, "batched lattices must share the g storage");
         for (int par = 0; par < 2; ++par) {
@@ -1377,7 +1372,7 @@ static int run_plan(BatchPlan &plan, int nsteps, cudaStream_t st)
         const BatchEntry *E = plan.entries[s & 1];
         int fp16 = plan.ctxs[0]->p.g_fp16;
         if (D == 2) {
-            Launch<2>::step_batch(E, plan.tiles, plan.ntiles, fp16, any_big(plan.ctxs), st);
+            Launch<2>::step_batch(E, plan.tiles, plan.ntiles, fp16, plan.big, st);
         } else {
             Launch<3>::moments_batch(E, plan.tiles, plan.ntiles, fp16, st);
             Launch<3>::step_batch(E, plan.tiles, plan.ntiles, fp16, false, st);
@@ -1418,6 +1413,7 @@ struct tlb_batch {
     std::vector<tlb_ctx *> ctxs;
     std::vector<int> base_cur;          // each context's buffer parity when the entries were written
     int D = 2, fp16 = 0;
+    bool big = false;                   // one of the lattices is a big_lattice
     cudaStream_t st = nullptr;          // the stream of ctxs[0]
     cudaStream_t cap = nullptr;         // private stream for graph capture and tuning
     std::vector<Block> owned;
@@ -1502,7 +1498,7 @@ static void batch_issue(const tlb_batch *b, int par, cudaStream_t st)
 {
     const BatchEntry *E = b->entries[par];
     if (b->D == 2) {
-        Launch<2>::step_batch(E, b->tiles, b->ntiles, b->fp16, any_big(b->ctxs), st, b->cfg.variant);
+        Launch<2>::step_batch(E, b->tiles, b->ntiles, b->fp16, b->big, st, b->cfg.variant);
     } else {
         Launch<3>::moments_batch(E, b->tiles, b->ntiles, b->fp16, st);
         Launch<3>::step_batch(E, b->tiles, b->ntiles, b->fp16, false, st, b->cfg.variant);
@@ -1553,6 +1549,7 @@ extern "C" int tlb_batch_create(tlb_ctx *const *ctxs, int n, const tlb_batch_con
     b->ctxs.assign(ctxs, ctxs + n);
     b->D = ctxs[0]->D;
     b->fp16 = ctxs[0]->p.g_fp16;
+    for (int k = 0; k < n; ++k) b->big |= big_lattice(ctxs[k]->N);
     b->st = ctxs[0]->stream;
     b->cfg = c;
     b->cfg.us_per_step = 0.0;
