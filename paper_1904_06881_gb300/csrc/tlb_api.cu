@@ -393,7 +393,6 @@ static DevParams make_dev(const tlb_params &p, const tlb_derived &d)
     q.ny = p.ny;
     q.nz = p.nz;
     q.N = (long long)p.nx * p.ny * p.nz;
-    q.lam1 = (float)p.lambda[0];
     q.hl1 = (float)(0.5 * p.lambda[0]);
     q.lam2 = (float)p.lambda[1];
     q.lam3 = (float)p.lambda[2];

@@ -135,58 +135,6 @@ __device__ __forceinline__ T *elem(T *base, int idx)
     return reinterpret_cast<T *>(reinterpret_cast<C *>(base) + (unsigned)idx * (unsigned)sizeof(T));
 }
 
-// ---------------------------------------------------------------------------
-// Thermodynamics (Sec. II.A-B), FP32
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ float gpoly(float x) { return x * (x - 0.5f) * (x - 1.0f); }
-
-struct Bulk {
-    float murB, mupB, p0;
-};
-
-// Bulk chemical potentials and pressure at (rho, phi): Eqs. BulkEnergy,
-// bulkchempotrho (lambda_2 term with the sign of the derivative of
-// Eq. BulkEnergy), bulkchempotphi, bulkpressure, with the Carnahan-Starling
-// Psi of Eq. PsiEOS and its printed derivative.
-__device__ __forceinline__ Bulk bulk_terms(const DevParams &p, float rho, float phi)
-{
-    const float C1 = (rho - p.rho_l) * p.inv_rgl;            // (rho - rho_l)/(rho_g - rho_l)
-    const float C2 = 0.5f * (fmaf(phi, p.inv_chi, 1.0f) - C1);
-    const float C3 = 0.5f * (fmaf(-phi, p.inv_chi, 1.0f) - C1);
-    float br = p.b * rho;
-    float psi, dpsi;
-    if (p.eos == 0) {
-        // Carnahan-Starling, Eq. PsiEOS and its printed derivative
-        float q = br - 4.0f;
-        float lr = __logf(rho);
-        psi = rho * fmaf(p.RT, lr, fmaf(-p.a, rho, p.C) - 8.0f * p.RT * (br - 6.0f) / (q * q));
-        dpsi = fmaf(p.RT, 1.0f + lr, fmaf(-2.0f * p.a, rho, p.C)) + 16.0f * p.RT * (br - 12.0f) / (q * q * q);
-    } else {
-        // van der Waals: Psi = rho (C - a rho + RT ln(rho/(1 - b rho)));
-        // Peng-Robinson adds - a A/(2 sqrt2 b) ln((b rho + sqrt2 - 1)/(sqrt2 + 1 - b rho))
-        // inside the bracket in place of - a rho (a A: p.aA)
-        const float om = 1.0f - br;
-        const float lg = __logf(rho / om);
-        if (p.eos == 1) {
-            psi = rho * (p.C - p.a * rho + p.RT * lg);
-            dpsi = p.C - 2.0f * p.a * rho + p.RT * lg + p.RT / om;
-        } else {
-            const float k = p.aA * (0.35355339f / p.b);      // a A / (2 sqrt2 b)
-            const float L = __logf((br + 0.41421356f) / (2.41421356f - br));
-            psi = rho * (p.C + p.RT * lg - k * L);
-            dpsi = p.C + p.RT * lg + p.RT / om - k * L - p.aA * rho / (1.0f + 2.0f * br - br * br);
-        }
-    }
-    float g2 = gpoly(C2), g3 = gpoly(C3);
-    const float s2 = fmaf(-C2, C2, C2), s3 = fmaf(-C3, C3, C3);
-    float fb = fmaf(p.hl1, psi - p.Psi0, fmaf(0.5f * p.lam2 * s2, s2, 0.5f * p.lam3 * s3 * s3));
-    Bulk r;
-    r.murB = fmaf(p.hl1, dpsi, fmaf(p.lam2, g2, p.lam3 * g3) * p.inv_drho);
-    r.mupB = fmaf(p.lam2, g2, -(p.lam3 * g3)) * p.inv_chi;
-    r.p0 = fmaf(rho, r.murB, fmaf(phi, r.mupB, -fb));
-    return r;
-}
-
 // ELBM beta of a node: the fluid's beta, or with per-component viscosities
 // the beta of the concentration-weighted mean viscosity (concentrations
 // clipped to [0, 1]), nu = (1/beta - 1)/6.
@@ -199,28 +147,6 @@ __host__ __device__ __forceinline__ float local_beta(const DevParams &p, float r
     const float nu = fmaf(c1, p.nu[0], fmaf(c2, p.nu[1], c3 * p.nu[2])) / (c1 + c2 + c3);
     return 1.0f / fmaf(6.0f, nu, 1.0f);
 }
-
-// ---------------------------------------------------------------------------
-// Product-form equilibrium (Eqs. eqrho, A, B): per axis the three D1Q3
-// factors w(c) A(u) B(u)^c, c = 0, +1, -1.
-// ---------------------------------------------------------------------------
-struct Fac {
-    float f0, fp, fm;
-};
-
-__device__ __forceinline__ Fac eq_factors(float u)
-{
-    float s = sqrtf(fmaf(3.0f * u, u, 1.0f));
-    float A = 2.0f - s;
-    float B = fmaf(2.0f, u, s) / (1.0f - u);
-    Fac r;
-    r.f0 = (2.0f / 3.0f) * A;
-    r.fp = (1.0f / 6.0f) * A * B;
-    r.fm = (1.0f / 6.0f) * A / B;
-    return r;
-}
-
-__device__ __forceinline__ float fac_of(const Fac &f, int c) { return c == 0 ? f.f0 : (c > 0 ? f.fp : f.fm); }
 
 // phi(y) = (1 + y) ln(1 + y) - y given l = ln(1 + y), accurate for small |y|
 // (series y^2/2 - y^3/6 + ...)

@@ -27,7 +27,7 @@ enum { TLB_WET_FORCE_ = 0 };
 struct DevParams {
     int nx, ny, nz;
     long long N;
-    float lam1, lam2, lam3;
+    float lam2, lam3;
     float chi, inv_chi;
     float a, b, RT, C, Psi0;
     float b4, hl1;       // b/4, lam1/2

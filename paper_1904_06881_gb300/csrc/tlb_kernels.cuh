@@ -284,76 +284,6 @@ __global__ void __launch_bounds__(128) ghost_kernel(DevParams p, const uint8_t *
     ghost_node<D>(p, type, rho, phi, ghosts[k]);
 }
 
-// ---------------------------------------------------------------------------
-// Node thermodynamics from a shared-memory tile of rho, phi (halo 2).
-// ---------------------------------------------------------------------------
-template <int D>
-struct Thermo {
-    float gr[3], gp[3], lr, lp;
-    Bulk b;
-    float mur, mup;
-    float P[6];     // xx yy zz xy xz yz
-};
-
-template <int D, int RX, int RY>
-__device__ __forceinline__ Thermo<D> node_thermo(const DevParams &p, const float2 *srp, int hx,
-                                                 int hy, int hz)
-{
-    constexpr int Q = Lat<D>::Q;
-    Thermo<D> t;
-    int c0 = hx + RX * (hy + RY * hz);
-    const float2 m0 = srp[c0];
-    float r0 = m0.x, p0v = m0.y;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) { t.gr[a] = 0.f; t.gp[a] = 0.f; }
-    t.lr = 0.f;
-    t.lp = 0.f;
-    // grad Q = 3 sum w_i c_i Q(x + c_i); lap Q = 6 sum w_i (Q(x + c_i) - Q(x))
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-        int m = (hx + cc<D>(i, 0)) + RX * ((hy + cc<D>(i, 1)) + RY * (hz + cc<D>(i, 2)));
-        const float2 mm = srp[m];
-        float rm = mm.x, pm = mm.y;
-        float w3 = 3.0f * wt<D>(i);
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            if (cc<D>(i, a) != 0) {
-                t.gr[a] = fmaf((float)cc<D>(i, a) * w3, rm, t.gr[a]);
-                t.gp[a] = fmaf((float)cc<D>(i, a) * w3, pm, t.gp[a]);
-            }
-        }
-        t.lr = fmaf(2.0f * w3, rm - r0, t.lr);
-        t.lp = fmaf(2.0f * w3, pm - p0v, t.lp);
-    }
-    t.b = bulk_terms(p, r0, p0v);
-    t.mur = fmaf(-p.krp, t.lp, fmaf(-p.krr, t.lr, t.b.murB));
-    t.mup = fmaf(-p.krp, t.lr, fmaf(-p.kpp, t.lp, t.b.mupB));
-    float g2r = 0.f, g2p = 0.f, grp = 0.f;
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        g2r += t.gr[a] * t.gr[a];
-        g2p += t.gp[a] * t.gp[a];
-        grp += t.gr[a] * t.gp[a];
-    }
-    float iso = t.b.p0 - p.krr * (r0 * t.lr + 0.5f * g2r) - p.kpp * (p0v * t.lp + 0.5f * g2p) -
-                p.krp * (r0 * t.lp + p0v * t.lr + grp);
-    constexpr int pa[6] = {0, 1, 2, 0, 0, 1}, pb[6] = {0, 1, 2, 1, 2, 2};
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        int a = pa[k], b = pb[k];
-        float v = 0.f;
-        if (a < D && b < D) {
-            v = p.krr * t.gr[a] * t.gr[b] + p.kpp * t.gp[a] * t.gp[b] + p.krp * (t.gr[a] * t.gp[b] + t.gp[a] * t.gr[b]);
-            if (a == b) v += iso;
-        }
-        t.P[k] = v;
-    }
-    return t;
-}
-
-template <int D>
-__host__ __device__ constexpr int NQC() { return D == 2 ? 3 : 6; }
-
 // index into the Q-tensor components stored per node: 2D {xx, yy, xy}, 3D {xx, yy, zz, xy, xz, yz}
 template <int D>
 __device__ __forceinline__ int qcomp(int a, int b)
@@ -383,159 +313,81 @@ namespace tlb {
 
 // ---------------------------------------------------------------------------
 // Passes over given or current fields that are not steps (one CTA = one tile
-// of TX x TY x TZ nodes, rho and phi from the moment arrays): MODE_INIT writes
-// the populations of rho, phi and u_init; MODE_AUX the auxiliary fields.
+// of TX x TY x TZ nodes, rho and phi from the moment arrays, the step's functions
+// for all that a step computes too): MODE_INIT writes the populations of rho, phi
+// and u_init; MODE_AUX the auxiliary fields.
 // ---------------------------------------------------------------------------
 template <int D, typename GT, int MODE>
-__global__ void __launch_bounds__(256) field_kernel(DevParams p, float *__restrict__ f_out, void *g_out,
-                                                    const float *__restrict__ rho, const float *__restrict__ phi,
-                                                    const uint8_t *__restrict__ type, const float *__restrict__ u_init,
+__global__ void __launch_bounds__(256) field_kernel(const __grid_constant__ BatchEntry e, const float *__restrict__ u_init,
                                                     AuxOut aux)
 {
     using S = StepShared<D>;
-    constexpr int Q = Lat<D>::Q;
-    constexpr int TX = S::TX, TY = S::TY, NT = S::NT, RX = S::RX, RY = S::RY, SX = S::SX, SY = S::SY;
-    constexpr int NR = S::NR, NS = S::NS, HZ2 = D == 3 ? 2 : 0, HZ1 = D == 3 ? 1 : 0;
-    constexpr int NC = NQC<D>();
-    __shared__ float2 srp[NR];            // rho, phi of the tile + halo 2
-    __shared__ float sQ[NC][NS];          // Q = rho c_s^2 I - P of the tile + halo 1
-    __shared__ float smu[NS];
-    __shared__ uint8_t stype[NS], srt[NR];
+    constexpr int Q = Lat<D>::Q, NPOS = Lat<D>::NPOS;
+    constexpr int TX = S::TX, TY = S::TY, RY = S::RY, SX = S::SX, SY = S::SY, HZ = D == 3 ? 1 : 0;
+    __shared__ S sh;
+    const DevParams &p = e.p;
+    const int tid = threadIdx.x;
     int x0, y0, z0;
     tile_origin<D>(p, blockIdx.x, x0, y0, z0);
-    const int tid = threadIdx.x;
-    // rho, phi and flags of the tile + halo 2, all of a thread's slots loaded
-    // in one round, then the ghost layer of Sec. IV
-    constexpr int PER = (NR + NT - 1) / NT;
-    float lr[PER], lp[PER];
-    uint8_t lt[PER];
-    bool ghost = false;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        const int k = tid + NT * j;
-        const int X = x0 - 2 + k % RX, Y = y0 - 2 + (k / RX) % RY, Z = z0 - HZ2 + k / (RX * RY);
-        const bool in = k < NR && X < p.nx + 2 && Y < p.ny + 2 && Z < p.nz + 2;
-        const int n = in ? node_near(p, X, Y, Z) : 0;
-        lt[j] = in ? __ldg(type + n) : (uint8_t)TLB_SOLID;
-        lr[j] = in ? __ldg(rho + n) : 0.f;
-        lp[j] = in ? __ldg(phi + n) : 0.f;
-    }
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        const int k = tid + NT * j;
-        if (k >= NR) break;
-        srt[k] = lt[j];
-        srp[k] = make_float2(lr[j], lp[j]);
-        ghost |= (lt[j] & TLB_GHOST) != 0;
-    }
-    if (ghost) {
-        const NodesGlobal acc{p, type, rho, phi};
-#pragma unroll 1
-        for (int k = tid; k < NR; k += NT) {
-            if (!(srt[k] & TLB_GHOST)) continue;      // unfilled slots hold TLB_SOLID alone
-            float gr, gp;
-            ghost_value<D>(p, acc, x0 - 2 + k % RX, y0 - 2 + (k / RX) % RY, z0 - HZ2 + k / (RX * RY), gr, gp);
-            srp[k] = make_float2(gr, gp);
-        }
-    }
-    __syncthreads();
-
-    for (int k = tid; k < NS; k += NT) {
-        const int lx = k % SX, ly = (k / SX) % SY, lz = k / (SX * SY);
-        const int X = x0 - 1 + lx, Y = y0 - 1 + ly, Z = z0 - HZ1 + lz;
-        const int c = (lx + 1) + RX * ((ly + 1) + RY * (lz + HZ1));
-        const uint8_t tk = (X >= p.nx + 1 || Y >= p.ny + 1 || Z >= p.nz + 1) ? (uint8_t)TLB_SOLID : srt[c];
-        stype[k] = tk;
-        if (tk & TLB_SOLID) {
-#pragma unroll
-            for (int j = 0; j < NC; ++j) sQ[j][k] = 0.f;
-            smu[k] = 0.f;
-            continue;
-        }
-        const Thermo<D> t = node_thermo<D, RX, RY>(p, srp, lx + 1, ly + 1, lz + HZ1);
-        const float cs2 = srp[c].x * (1.0f / 3.0f);
-        if constexpr (D == 2) {
-            sQ[0][k] = cs2 - t.P[0];
-            sQ[1][k] = cs2 - t.P[1];
-            sQ[2][k] = -t.P[3];
-        } else {
-#pragma unroll
-            for (int j = 0; j < 6; ++j) sQ[j][k] = (j < 3 ? cs2 : 0.f) - t.P[j];
-        }
-        smu[k] = t.mup;
-    }
+    gather_moments<D, true>(e, x0, y0, z0, sh, [] {});
+    tensor_stage<D, true>(p, x0, y0, z0, sh);
     __syncthreads();
 
     // one node per thread
     const int tx = tid % TX, ty = (tid / TX) % TY, tz = tid / (TX * TY);
     const int x = x0 + tx, y = y0 + ty, z = z0 + tz;
     if (x >= p.nx || y >= p.ny || z >= p.nz) return;
-    const int sx = tx + 1, sy = ty + 1, sz = tz + HZ1;
-    const int sc = sx + SX * (sy + SY * sz);
-    const uint8_t tc = stype[sc];
+    const int sc = (tx + 1) + SX * ((ty + 1) + SY * (tz + HZ));
+    const uint8_t tc = sh.type[sc];
     if (tc & TLB_SOLID) return;
     const int n = x + p.nx * (y + p.ny * z);
-    const float2 rph = srp[(sx + 1) + RX * ((sy + 1) + RY * (sz + HZ1))];
-    const float r = rph.x, ph = rph.y;
-    // force F = div(rho c_s^2 I - P) with the wall rules, and the wetting force of method 1
-    float F[3] = {0.f, 0.f, 0.f};
-    auto qc = [&](int c, int m) { return sQ[c][m]; };
-    if (!(tc & TLB_FIRST)) {
+    const float2 *c = sh.rp + (tx + 2) + S::PX * ((ty + 2) + RY * (tz + 2 * HZ));
+    const float r = c->x, ph = c->y;
+    float F[D];
+    const float mup = node_force<D, true>(p, sh, sc, tc, r, ph, F);
+    if constexpr (MODE == MODE_AUX) {
+        const Stress<D> s = node_stress<D, S::PX, RY>(p, c);
+        if (aux.p0) aux.p0[n] = s.p0;
+        if (aux.mur) aux.mur[n] = fmaf(-p.krp, s.lap.y, fmaf(-p.krr, s.lap.x, bulk_mur(p, r, ph)));
+        if (aux.mup) aux.mup[n] = s.mup;
 #pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            const int m = sc + cc<D>(i, 0) + SX * (cc<D>(i, 1) + SY * cc<D>(i, 2));
-#pragma unroll
-            for (int a = 0; a < D; ++a) {
-                float acc = 0.f;
-#pragma unroll
-                for (int b = 0; b < D; ++b)
-                    if (cc<D>(i, b) != 0) acc += (float)cc<D>(i, b) * sQ[qcomp<D>(a, b)][m];
-                F[a] = fmaf(3.0f * wt<D>(i), acc, F[a]);
-            }
-        }
-    } else {
-        wall_force<D>(qc, stype, tc, sc, F);
-    }
-    wetting_force<D>(p, stype, tc, sc, r, ph, F);
-    if (MODE == MODE_AUX) {
-        const Thermo<D> t = node_thermo<D, RX, RY>(p, srp, sx + 1, sy + 1, sz + HZ1);
-        if (aux.p0) aux.p0[n] = t.b.p0;
-        if (aux.mur) aux.mur[n] = t.mur;
-        if (aux.mup) aux.mup[n] = t.mup;
         for (int a = 0; a < 3; ++a)
-            if (aux.F[a]) aux.F[a][n] = (a < D) ? F[a] : 0.f;
-        for (int j = 0; j < 6; ++j)
-            if (aux.P[j]) aux.P[j][n] = t.P[j];
-        return;
+            if (aux.F[a]) aux.F[a][n] = a < D ? F[a < D ? a : 0] : 0.f;
+#pragma unroll
+        for (int j = 0; j < 6; ++j)        // xx yy zz xy xz yz
+            if (aux.P[j]) aux.P[j][n] = D == 3 ? (j < 3 ? s.iso + s.d[j] : s.o[j - 3])
+                                               : j < 2 ? s.iso + s.d[j] : j == 2 ? s.iso : j == 3 ? s.o[0] : 0.f;
+    } else {
+        // f = f^eq(rho, v - F/(2 rho)), g = g^eq(phi, v, mu_phi) at the node itself
+        const float inv_r = 1.0f / r;
+        float v[D], f0[D], fp[D], fm[D], rest = r;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            v[a] = u_init ? u_init[(long long)a * p.N + n] : 0.f;
+            const float u = fmaf(-0.5f * F[a], inv_r, v[a]);
+            const Fac2 t = eq_factors2<D>(f2(u, u));
+            f0[a] = t.f0.x;
+            fp[a] = t.fp.x;
+            fm[a] = t.fm.x;
+            rest *= f0[a];
+        }
+        float2 eq[NPOS];
+        equilibria<D>(r, f0, fp, fm, eq);
+        const GEq ge = g_eq<D>(p, ph, mup, v);
+        float2 gsum = f2(0.f, 0.f);
+        e.f_out[n] = rest - wt<D>(0);
+#pragma unroll
+        for (int k = 0; k < NPOS; ++k) {
+            const float w = wt<D>(2 * k + 1);
+            const float2 gk = ge.pair(w, along<D>(k, v));
+            gsum = add2(gsum, gk);
+            e.f_out[(long long)(2 * k + 1) * p.N + n] = eq[k].x - w;
+            e.f_out[(long long)(2 * k + 2) * p.N + n] = eq[k].y - w;
+            GIO<GT>::st(e.g_out, 2 * k + 1, n, gk.x, p);
+            GIO<GT>::st(e.g_out, 2 * k + 2, n, gk.y, p);
+        }
+        GIO<GT>::st(e.g_out, 0, n, ph - (gsum.x + gsum.y), p);
     }
-    // f = f^eq(rho, v - F/(2 rho)), g = g^eq(phi, v, mu_phi) at the node itself
-    const float inv_r = 1.0f / r, mup = smu[sc];
-    float v[3] = {0.f, 0.f, 0.f};
-    Fac fu[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        v[a] = u_init ? u_init[(long long)a * p.N + n] : 0.f;
-        fu[a] = eq_factors(v[a] - 0.5f * F[a] * inv_r);
-    }
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        float e = r;
-#pragma unroll
-        for (int a = 0; a < D; ++a) e *= fac_of(fu[a], cc<D>(i, a));
-        f_out[(long long)i * p.N + n] = e - wt<D>(i);
-    }
-    const float v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    float gsum = 0.f;
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-        float cv = 0.f;
-#pragma unroll
-        for (int a = 0; a < D; ++a) cv += (float)cc<D>(i, a) * v[a];
-        const float ge = wt<D>(i) * (3.0f * p.Gamma * mup + 3.0f * ph * cv + 4.5f * ph * cv * cv - 1.5f * ph * v2);
-        gsum += ge;
-        GIO<GT>::st(g_out, i, n, ge, p);
-    }
-    GIO<GT>::st(g_out, 0, n, ph - gsum, p);
 }
 
 // ---------------------------------------------------------------------------
@@ -674,14 +526,16 @@ void Launch<D>::field_pass(const DevParams &p, const DevState &s, int mode, cons
 {
     // one dimension: the others end at 65535, which a lattice of many tile rows passes
     const int grid = tiles(p), block = Tile<D>::X * Tile<D>::Y * Tile<D>::Z;
-    float *f = s.f[s.cur];
-    void *g = s.g[s.cur];
-    if (mode == MODE_AUX)
-        field_kernel<D, float, MODE_AUX><<<grid, block, 0, st>>>(p, f, g, s.rho, s.phi, s.type, nullptr, aux);
-    else if (p.g_fp16)
-        field_kernel<D, __half, MODE_INIT><<<grid, block, 0, st>>>(p, f, g, s.rho, s.phi, s.type, u_init, aux);
-    else
-        field_kernel<D, float, MODE_INIT><<<grid, block, 0, st>>>(p, f, g, s.rho, s.phi, s.type, u_init, aux);
+    BatchEntry e = {};
+    e.p = p;
+    e.f_out = s.f[s.cur];
+    e.g_out = s.g[s.cur];
+    e.rho = s.rho;
+    e.phi = s.phi;
+    e.type = s.type;
+    if (mode == MODE_AUX) field_kernel<D, float, MODE_AUX><<<grid, block, 0, st>>>(e, nullptr, aux);
+    else if (p.g_fp16) field_kernel<D, __half, MODE_INIT><<<grid, block, 0, st>>>(e, u_init, aux);
+    else field_kernel<D, float, MODE_INIT><<<grid, block, 0, st>>>(e, u_init, aux);
 }
 
 template <int D>

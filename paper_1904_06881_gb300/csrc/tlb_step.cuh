@@ -90,14 +90,52 @@ __device__ __forceinline__ float bulk_p0(const DevParams &p, float rho, float ph
     return fmaf(p.hl1, eos_pressure(p, rho) + p.Psi0, -v);
 }
 
-// Q = rho c_s^2 I - P ({xx, yy, xy} in 2D, {xx, yy, zz, xy, xz, yz} in 3D) and
-// mu_phi at the node whose (rho, phi) is c[0] in a region of row length RX and
-// RY rows per plane.  The stencils (grad Q = 3 sum w_i c_i Q(x + c_i), lap Q =
+// The bulk part of mu_rho (Eq. bulkchempotrho, the lambda_2 term with the sign of
+// the derivative of Eq. BulkEnergy), an auxiliary field that no step needs: the one
+// place of the logarithm of Psi, through Psi' as printed for Carnahan-Starling
+// (Eq. PsiEOS), and with Psi = rho (C - a rho + RT ln(rho/(1 - b rho))) of van der
+// Waals, where Peng-Robinson has - a A/(2 sqrt2 b) ln((b rho + sqrt2 - 1)/(sqrt2 +
+// 1 - b rho)) in place of - a rho (a A: p.aA).
+__device__ __forceinline__ float bulk_mur(const DevParams &p, float rho, float phi)
+{
+    const float br = p.b * rho;
+    float dpsi;
+    if (p.eos == 0) {
+        const float q = br - 4.0f;
+        dpsi = fmaf(p.RT, 1.0f + logf(rho), fmaf(-2.0f * p.a, rho, p.C)) + 16.0f * p.RT * (br - 12.0f) / (q * q * q);
+    } else {
+        const float om = 1.0f - br, lg = logf(rho / om);
+        if (p.eos == 1) {
+            dpsi = fmaf(p.RT, lg, fmaf(-2.0f * p.a, rho, p.C)) + p.RT / om;
+        } else {
+            const float k = p.aA * (0.35355339f / p.b);      // a A / (2 sqrt2 b)
+            const float L = logf((br + 0.41421356f) / (2.41421356f - br));
+            dpsi = fmaf(p.RT, lg, fmaf(-k, L, p.C)) + p.RT / om - p.aA * rho / fmaf(br, 2.0f - br, 1.0f);
+        }
+    }
+    const float C1 = (rho - p.rho_l) * p.inv_rgl, a = phi * p.inv_chi;
+    const float h = fmaf(-0.5f, C1, 0.5f);
+    const float C2 = fmaf(0.5f, a, h), C3 = fmaf(-0.5f, a, h);
+    const float g2 = C2 * (C2 - 0.5f) * (C2 - 1.0f), g3 = C3 * (C3 - 0.5f) * (C3 - 1.0f);
+    return fmaf(p.hl1, dpsi, fmaf(p.lam2, g2, p.lam3 * g3) * p.inv_drho);
+}
+
+// Pressure tensor P = iso I + {d on the diagonal, o = xy, xz, yz off it}, p_0,
+// mu_phi and the Laplacians of (rho, phi)
+template <int D>
+struct Stress {
+    float iso, d[D], o[D == 3 ? 3 : 1], p0, mup;
+    float2 lap;
+};
+
+// The pressure tensor and mu_phi at the node whose (rho, phi) is c[0] in a region
+// of row length RX and RY rows per plane.  The stencils (grad Q = 3 sum w_i c_i Q(x + c_i), lap Q =
 // 6 sum w_i (Q(x + c_i) - Q(x))) as products of (1, 4, 1)/6 and (-1, 0, 1)/6
 // along the axes, on differences to the node itself.
 template <int D, int RX, int RY>
-__device__ __forceinline__ void node_q(const DevParams &p, const float2 *__restrict__ c, float *q, float &mup)
+__device__ __forceinline__ Stress<D> node_stress(const DevParams &p, const float2 *__restrict__ c)
 {
+    Stress<D> s;
     const float2 m0 = c[0];
     const float2 four = f2(4.0f, 4.0f);
     float2 g[D], lap;
@@ -138,9 +176,10 @@ __device__ __forceinline__ void node_q(const DevParams &p, const float2 *__restr
         lap = mul2(fma2(four, S[1], add2(S[0], S[2])), f2(1.0f / 6.0f, 1.0f / 6.0f));
     }
     float mupB;
-    const float p0 = bulk_p0(p, m0.x, m0.y, mupB);
+    s.p0 = bulk_p0(p, m0.x, m0.y, mupB);
+    s.lap = lap;
     const float Lr = fmaf(p.krr, lap.x, p.krp * lap.y), Lp = fmaf(p.kpp, lap.y, p.krp * lap.x);
-    mup = mupB - Lp;
+    s.mup = mupB - Lp;
     // P_ab = krr dr_a dr_b + kpp dp_a dp_b + krp (dr_a dp_b + dp_a dr_b) + iso delta_ab,
     // iso = p0 - rho Lr - phi Lp - (trace of the gradient part)/2
     float hr[D], hp[D];
@@ -150,23 +189,33 @@ __device__ __forceinline__ void node_q(const DevParams &p, const float2 *__restr
         hp[a] = fmaf(p.kpp, g[a].y, p.krp * g[a].x);
     }
     auto gg = [&](int a, int b) { return fmaf(g[a].x, hr[b], g[a].y * hp[b]); };
-    float d[D], tr = 0.f;
+    float tr = 0.f;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        d[a] = gg(a, a);
-        tr += d[a];
+        s.d[a] = gg(a, a);
+        tr += s.d[a];
     }
-    const float iso = fmaf(-0.5f, tr, fmaf(-m0.y, Lp, fmaf(-m0.x, Lr, p0)));
-    const float base = fmaf(m0.x, 1.0f / 3.0f, -iso);
-#pragma unroll
-    for (int a = 0; a < D; ++a) q[a] = base - d[a];
+    s.iso = fmaf(-0.5f, tr, fmaf(-m0.y, Lp, fmaf(-m0.x, Lr, s.p0)));
+    s.o[0] = gg(0, 1);
     if constexpr (D == 3) {
-        q[3] = -gg(0, 1);
-        q[4] = -gg(0, 2);
-        q[5] = -gg(1, 2);
-    } else {
-        q[2] = -gg(0, 1);
+        s.o[1] = gg(0, 2);
+        s.o[2] = gg(1, 2);
     }
+    return s;
+}
+
+// Q = rho c_s^2 I - P ({xx, yy, xy} in 2D, {xx, yy, zz, xy, xz, yz} in 3D) and
+// mu_phi there
+template <int D, int RX, int RY>
+__device__ __forceinline__ void node_q(const DevParams &p, const float2 *__restrict__ c, float *q, float &mup)
+{
+    const Stress<D> s = node_stress<D, RX, RY>(p, c);
+    const float base = fmaf(c[0].x, 1.0f / 3.0f, -s.iso);
+#pragma unroll
+    for (int a = 0; a < D; ++a) q[a] = base - s.d[a];
+#pragma unroll
+    for (int k = 0; k < (D == 3 ? 3 : 1); ++k) q[D + k] = -s.o[k];
+    mup = s.mup;
 }
 
 // ---------------------------------------------------------------------------
@@ -510,17 +559,18 @@ __device__ __forceinline__ void own_copies_3d(const BatchEntry &e, int x0, int y
 
 // Stage A of a D3Q27 tile: rho, phi (and flags) of the tile + halo 2 from the
 // moments pass, own_copies() called behind those loads (copies requested ahead
-// of them would keep them waiting), and in tiles at walls the ghost layer (the moments pass leaves ghost
-// nodes alone).
-template <bool WALLS, class OWN>
-__device__ __forceinline__ void gather_3d(const BatchEntry &e, int x0, int y0, int z0, StepShared<3> &sh,
-                                          const OWN &own_copies)
+// of them would keep them waiting), and in tiles at walls the ghost layer (the
+// moments pass leaves ghost nodes alone).  Also the D2Q9 tiles of the field pass.
+template <int D, bool WALLS, class OWN>
+__device__ __forceinline__ void gather_moments(const BatchEntry &e, int x0, int y0, int z0, StepShared<D> &sh,
+                                               const OWN &own_copies)
 {
-    using S = StepShared<3>;
-    constexpr int NT = S::NT, RX = S::RX, RY = S::RY, RZ = S::RZ, NR = S::NR, TX = S::TX, TY = S::TY;
+    using S = StepShared<D>;
+    constexpr int NT = S::NT, RX = S::RX, RY = S::RY, NR = S::NR, HZ = D == 3 ? 2 : 0;
     const DevParams &p = e.p;
     const int tid = threadIdx.x;
-    if constexpr (!WALLS) {
+    if constexpr (D == 3 && !WALLS) {
+        constexpr int RZ = S::RZ, TX = S::TX, TY = S::TY;
         // the region of a tile away from the lattice's edges lies in memory as
         // rows of RX nodes: two nodes a load where the rows are 8-byte aligned
         if (x0 >= 2 && y0 >= 2 && z0 >= 2 && x0 + TX + 2 <= p.nx && y0 + TY + 2 <= p.ny &&
@@ -559,8 +609,8 @@ __device__ __forceinline__ void gather_3d(const BatchEntry &e, int x0, int y0, i
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         const int k = tid + NT * j;
-        const int X = x0 - 2 + k % RX, Y = y0 - 2 + (k / RX) % RY, Z = z0 - 2 + k / (RX * RY);
-        const bool in = k < NR && X < p.nx + 2 && Y < p.ny + 2 && Z < p.nz + 2;
+        const int X = x0 - 2 + k % RX, Y = y0 - 2 + (k / RX) % RY, Z = z0 - HZ + k / (RX * RY);
+        const bool in = k < NR && X < p.nx + 2 && Y < p.ny + 2 && Z < p.nz + HZ;
         const int n = in ? node_near(p, X, Y, Z) : 0;
         if (WALLS) lt[j] = in ? __ldg(e.type + n) : (uint8_t)TLB_SOLID;
         lr[j] = in ? e.rho[n] : 0.f;
@@ -583,7 +633,7 @@ __device__ __forceinline__ void gather_3d(const BatchEntry &e, int x0, int y0, i
         for (int k = tid; k < NR; k += NT) {
             if (!(sh.rtype[k] & TLB_GHOST)) continue;      // unfilled slots hold TLB_SOLID alone
             float gr, gp;
-            ghost_value<3>(p, acc, x0 - 2 + k % RX, y0 - 2 + (k / RX) % RY, z0 - 2 + k / (RX * RY), gr, gp);
+            ghost_value<D>(p, acc, x0 - 2 + k % RX, y0 - 2 + (k / RX) % RY, z0 - HZ + k / (RX * RY), gr, gp);
             sh.rp[(k / RX) * S::PX + k % RX] = make_float2(gr, gp);
         }
     }
@@ -967,8 +1017,38 @@ __device__ __forceinline__ void push_f(const BatchEntry &e, const Push<D> &to, u
     }
 }
 
-// LBGK of g (Eq. CahnHilliardLBM) with g^eq(phi, v, mu_phi), pushed like f.
-// g^eq_i = w_i (gA + gB c.v + gC (c.v)^2): an even and an odd part per pair.
+// c.v of the pair k's first direction
+template <int D>
+__device__ __forceinline__ float along(int k, const float (&v)[D])
+{
+    float cv = 0.f;
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+        if (Lat<D>::pos(k, a) != 0) cv += Lat<D>::pos(k, a) > 0 ? v[a] : -v[a];
+    return cv;
+}
+
+// g^eq(phi, v, mu_phi): g^eq_i = w_i (A + B c.v + C (c.v)^2), an even and an odd
+// part per pair
+struct GEq {
+    float A, B, C;
+    __device__ __forceinline__ float2 pair(float w, float cv) const
+    {
+        const float ev = fmaf((w * C) * cv, cv, w * A), od = w * B;
+        return f2(fmaf(od, cv, ev), fmaf(-od, cv, ev));
+    }
+};
+
+template <int D>
+__device__ __forceinline__ GEq g_eq(const DevParams &p, float ph, float mup, const float (&v)[D])
+{
+    float v2 = 0.f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) v2 = fmaf(v[a], v[a], v2);
+    return {fmaf(3.0f * p.Gamma, mup, -(1.5f * ph * v2)), 3.0f * ph, 4.5f * ph};
+}
+
+// LBGK of g (Eq. CahnHilliardLBM) with g^eq(phi, v, mu_phi), pushed like f
 template <int D, typename GT, bool BB, bool BIG, class LD>
 __device__ __forceinline__ void relax_g(const BatchEntry &e, const Push<D> &to, unsigned solid_nb, float ph, float mup,
                                         const float (&v)[D], const LD &ld_g)
@@ -980,22 +1060,14 @@ __device__ __forceinline__ void relax_g(const BatchEntry &e, const Push<D> &to, 
         else if constexpr (sizeof(GT) == 4) *elem<BIG>((float *)e.g_out + (long long)i * p.N, m) = val;
         else *elem<BIG>((__half *)((char *)e.g_out + 4 * p.N) + (long long)(i - 1) * p.N, m) = __float2half_rn(val * p.g_scale);
     };
-    float v2 = 0.f;
-#pragma unroll
-    for (int a = 0; a < D; ++a) v2 = fmaf(v[a], v[a], v2);
-    const float gA = fmaf(3.0f * p.Gamma, mup, -(1.5f * ph * v2)), gB = 3.0f * ph, gC = 4.5f * ph;
+    const GEq eq = g_eq<D>(p, ph, mup, v);
     const float2 itau = f2(p.inv_tau_g, p.inv_tau_g);
     float2 gsum = f2(0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < Lat<D>::NPOS; ++k) {
         const float w = wt<D>(2 * k + 1);
         const float2 gi = f2(ld_g(2 * k + 1), ld_g(2 * k + 2));
-        float cv = 0.f;
-#pragma unroll
-        for (int a = 0; a < D; ++a)
-            if (Lat<D>::pos(k, a) != 0) cv += Lat<D>::pos(k, a) > 0 ? v[a] : -v[a];
-        const float ev = fmaf((w * gC) * cv, cv, w * gA), od = w * gB;
-        const float2 ge = f2(fmaf(od, cv, ev), fmaf(-od, cv, ev));
+        const float2 ge = eq.pair(w, along<D>(k, v));
         gsum = add2(gsum, ge);
         const float2 gn = fma2(sub2<D>(ge, gi), itau, gi);
         put(2 * k + 1, gn.x);
@@ -1020,7 +1092,7 @@ __device__ __forceinline__ void step_tile(const BatchEntry &e, int x0, int y0, i
     // tensor copies need the staging area 128-byte aligned (checked, uniform per CTA)
     const bool use_tma = D == 3 && e.tm[0] != nullptr && (smem_u32(stage) & 127u) == 0;
     if constexpr (D == 2) gather_2d<GT, WALLS, BIG>(e, x0, y0, sh, stage);
-    else gather_3d<WALLS>(e, x0, y0, z0, sh, [&] { own_copies_3d<GT>(e, x0, y0, z0, sh, stage, use_tma); });
+    else gather_moments<D, WALLS>(e, x0, y0, z0, sh, [&] { own_copies_3d<GT>(e, x0, y0, z0, sh, stage, use_tma); });
 
     tensor_stage<D, WALLS>(p, x0, y0, z0, sh);
     // every thread's staged copies complete before the barrier, so each thread
