@@ -241,7 +241,9 @@ long long tlb_launch_count(const tlb_ctx *ctx);
  * flags formed from them, when the lattice, the sizes, the mask's contents or the
  * stream differ from the previous call's on this device; otherwise the copy
  * in the array is used again (one N-byte comparison instead of the host pass
- * over the mask and its upload).  Calls that overlap on the GPU --
+ * over the mask and its upload).  On a stream that is being recorded into a graph
+ * only a call of that second kind is taken (else TLB_E_UNSUPPORTED: the upload's
+ * source is gone when the graph runs).  Calls that overlap on the GPU --
  * concurrent streams or host threads on one device -- race and must be
  * serialised by the caller.  Divergence is not reported by this call; use a
  * context (tlb_sync) to get it. */

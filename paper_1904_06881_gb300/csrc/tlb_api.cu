@@ -2114,6 +2114,11 @@ extern "C" int tlb_step_noalloc(const tlb_params *pin, const uint8_t *mask, floa
                 nd.nz == p->nz && nd.stream == st && (mask == nullptr) == nd.mask.empty() &&
                 (mask == nullptr || std::memcmp(mask, nd.mask.data(), (size_t)N) == 0);
     if (!same) {
+        // a recording would copy from this call's host arrays when they are gone, and
+        // later calls take its flags for those of the array
+        if (is_recording(st))
+            return fail(TLB_E_UNSUPPORTED, "tlb_step_noalloc: a call that is recorded into a graph needs the flags of its "
+                                           "geometry in place (the same call once before, nsteps = 0 will do)");
         nd.have_geom = false;
         std::vector<uint8_t> flags;
         std::vector<int> ghosts;

@@ -1,7 +1,7 @@
 """tlb_step on a stream that is recorded into a CUDA graph: the replayed steps
 take the solid mask that is set when they run, not the one of the recording,
 and a recording that has been invalidated refuses steps, which then do not
-count."""
+count.  tlb_step_noalloc is recorded with its geometry's flags in place only."""
 import ctypes
 
 import numpy as np
@@ -112,4 +112,52 @@ def test_steps_that_cannot_be_launched_do_not_count(lattice, phases):
     for a, b in zip(lat.populations(), ref.populations()):
         assert np.array_equal(a[:, fl], b[:, fl])
     lat.close()
+    ref.close()
+
+
+@pytest.mark.parametrize("lattice", [W.D2Q9, W.D3Q27])
+def test_recorded_allocation_free_steps(lattice):
+    import torch
+
+    from paper_1904_06881_gb300 import tlb
+
+    drv, wl, s = _Driver(), _wl(lattice, "block"), torch.cuda.Stream()
+    ref = tlb.lattice_from_workload(wl)
+    c, _ = tlb.tlb_lattice_directions(lattice)
+    w = np.ones(len(c), np.float32)            # the weights as the library forms them
+    for a in range(2 if lattice == W.D2Q9 else 3):
+        w = w * np.where(c[:, a] == 0, np.float32(2) / np.float32(3), np.float32(1) / np.float32(6))
+    w = w.astype(np.float64)[:, None]
+    f0, g0 = ref.populations()
+    f, g = (torch.tensor(v.astype(np.float32), device="cuda") for v in (f0 - w, g0))
+    f_tmp, g_tmp = torch.empty_like(f), torch.empty_like(g)
+    torch.cuda.synchronize()
+    p = tlb.make_params(lattice, wl["nx"], wl["ny"], wl["nz"], **wl["params"])
+
+    def call(nsteps):
+        tlb.tlb_step_noalloc(p, wl["mask"], f.data_ptr(), f_tmp.data_ptr(), g.data_ptr(), g_tmp.data_ptr(), nsteps,
+                             s.cuda_stream)
+
+    drv.begin(s.cuda_stream)
+    with pytest.raises(tlb.TlbError) as e:
+        call(3)
+    assert e.value.code == -4
+    rc, graph = drv.end(s.cuda_stream)         # the recording itself stays valid
+    assert rc == 0
+    drv.cu.cuGraphDestroy(graph)
+    call(0)
+    drv.begin(s.cuda_stream)
+    call(3)
+    rc, graph = drv.end(s.cuda_stream)
+    assert rc == 0
+    ex = drv.instantiate(graph)
+    fl = wl["mask"].reshape(-1) == 0
+    for _ in range(2):
+        drv.launch(ex, s.cuda_stream)
+        torch.cuda.synchronize()
+        ref.step(3)
+        fr, gr = ref.populations()
+        assert np.array_equal((f.double().cpu().numpy() + w)[:, fl], fr[:, fl])
+        assert np.array_equal(g.double().cpu().numpy()[:, fl], gr[:, fl])
+    drv.destroy(graph, ex)
     ref.close()
