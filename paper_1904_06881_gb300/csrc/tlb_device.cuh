@@ -201,7 +201,7 @@ __host__ __device__ __forceinline__ float alpha_series(float a2, float a3, float
 // 3.3e-9 at ALPHA_SHORT_MAX, a thirtieth of what rounding alpha = 2 + ... leaves
 // (half a unit in its last place, 1.2e-7 above 2 and 6e-8 below).  In FP32 the
 // root is then as far from the exact one as with all five terms (1.19e-7 at most,
-// 5.4e-8 on average); at 0.01 it was 3.4e-7 and 1.5e-7.  Steps with the limit at
+// 5.4e-8 on average); with the limit at 0.01 it is 3.5e-7 and 1.5e-7.  Steps with the limit at
 // 0.01, here, and without the short form: D2Q9 2048 x 2048 171.0, 171.2, 180.0 us,
 // D3Q27 192 x 192 x 128 746, 764, 764.
 constexpr float ALPHA_SHORT_MAX = 0.001f;

@@ -1,11 +1,17 @@
 // tlb_step.cuh -- the stepping kernel of the ternary ELBM (one CTA = one tile
 // of TX x TY x TZ nodes), templated on the dimension D.
 //
-// What bounds it: instruction issue.  The populations are read and written
-// once (16Q bytes a node), and the arithmetic of a node is large next to that:
-// stencils of rho, phi and of the pressure tensor, two product equilibria,
-// the entropic root, two relaxations.  So the arithmetic is written for few
-// instructions:
+// What bounds it: no one unit on large lattices.  The populations are read and
+// written once (16Q bytes a node), and the arithmetic of a node is large next to
+// that: stencils of rho, phi and of the pressure tensor, two product equilibria,
+// the entropic root, two relaxations.  D2Q9 issues in 0.6 of the cycles at 30
+// warps an SM (waits for loads, the shared-memory queue and the packed FP32 pipe),
+// D3Q27 in 0.47 (captured with cold caches; 0.55 over the time of a step) at the 14
+// that its registers and shared memory admit, where waits for instructions, for
+// loads, at barriers and for dependent results share the rest.  On lattices of one
+// wave a step is a tile's chain of stages, run once: instruction fetch is its largest
+// stall (5 warps an issue of 1024 x 64 with cold caches, loads 2).
+// So the arithmetic is written for few instructions:
 //   - opposite directions +c, -c form a pair held in a float2 and handled by
 //     the packed FP32 instructions (two results per issue);
 //   - (rho, phi) form another such pair in the stencils, which are applied one
@@ -17,10 +23,10 @@
 //     and bounce-back;
 //   - a lattice stepped alone passes its entry by value, so that parameters
 //     and array bases are constant-bank operands.
-// Warp instructions x 32 a node, with the former kernels' in brackets: D2Q9
-// 2048 x 2048 928 (1506), D3Q27 2556 (3876).  Kernel time: D2Q9 4096 x 4096 0.618
-// ms, 58 % of 6.8 TB/s (0.83 ms); D3Q27 192 x 192 x 128 0.537 ms, 57 % (0.77 ms),
-// where the chain of a tile's stages at 16 warps an SM is what is left.
+// Warp instructions x 32 a node: D2Q9 2048 x 2048 929, D3Q27 2563 (1506 and 3876
+// with directions one by one, flags in every tile and the entry in shared memory).
+// Kernel time: D2Q9 4096 x 4096 0.622 ms, 58 % of the measured 6.78 TB/s; D3Q27 192 x
+// 192 x 128 0.551 ms, 56 %.
 #pragma once
 #include "tlb_device.cuh"
 
@@ -508,53 +514,53 @@ __device__ __forceinline__ void own_copies_3d(const BatchEntry &e, int x0, int y
     constexpr int Q = 27, NT = StepShared<3>::NT, TX = StepShared<3>::TX, TY = StepShared<3>::TY;
     const DevParams &p = e.p;
     const int tid = threadIdx.x;
-            if (use_tma) {
-                // one thread: a box of TX x TY x TZ nodes x all directions per array
-                // (x0 is a multiple of 16 nodes: 16-byte aligned inner coordinate)
-                if (tid == 0) {
-                    mbar_init(&sh.tma_bar, 1);
-                    const unsigned bytes = (unsigned)(Q * NT * 4) +
-                                           (sizeof(GT) == 4 ? (unsigned)(Q * NT * 4) : (unsigned)(NT * 4 + (Q - 1) * NT * 2));
+    if (use_tma) {
+        // one thread: a box of TX x TY x TZ nodes x all directions per array
+        // (x0 is a multiple of 16 nodes: 16-byte aligned inner coordinate)
+        if (tid == 0) {
+            mbar_init(&sh.tma_bar, 1);
+            const unsigned bytes = (unsigned)(Q * NT * 4) +
+                                   (sizeof(GT) == 4 ? (unsigned)(Q * NT * 4) : (unsigned)(NT * 4 + (Q - 1) * NT * 2));
 #ifdef TLB_TEST_TMA_TIMEOUT
-                    // test builds only: the barrier expects 16 bytes more than the
-                    // copies send, so its wait runs out and the timeout path runs
-                    mbar_expect_tx(&sh.tma_bar, bytes + 16u);
+            // test builds only: the barrier expects 16 bytes more than the
+            // copies send, so its wait runs out and the timeout path runs
+            mbar_expect_tx(&sh.tma_bar, bytes + 16u);
 #else
-                    mbar_expect_tx(&sh.tma_bar, bytes);
+            mbar_expect_tx(&sh.tma_bar, bytes);
 #endif
-                    tma_load_4d(&stage[0], e.tm[0], x0, y0, z0, 0, &sh.tma_bar);
-                    if (sizeof(GT) == 4) {
-                        tma_load_4d(&stage[Q * NT], e.tm[1], x0, y0, z0, 0, &sh.tma_bar);
-                    } else {
-                        tma_load_3d(&stage[Q * NT], e.tm[1], x0, y0, z0, &sh.tma_bar);
-                        tma_load_4d(&stage[(Q + 1) * NT], e.tm[2], x0, y0, z0, 0, &sh.tma_bar);
-                    }
-                }
-                return;
+            tma_load_4d(&stage[0], e.tm[0], x0, y0, z0, 0, &sh.tma_bar);
+            if (sizeof(GT) == 4) {
+                tma_load_4d(&stage[Q * NT], e.tm[1], x0, y0, z0, 0, &sh.tma_bar);
+            } else {
+                tma_load_3d(&stage[Q * NT], e.tm[1], x0, y0, z0, &sh.tma_bar);
+                tma_load_4d(&stage[(Q + 1) * NT], e.tm[2], x0, y0, z0, 0, &sh.tma_bar);
             }
-            const int ax = x0 + tid % TX, ay = y0 + (tid / TX) % TY, az = z0 + tid / (TX * TY);
-            if (ax < p.nx && ay < p.ny && az < p.nz) {
-                const int an = ax + p.nx * (ay + p.ny * az);
+        }
+        return;
+    }
+    const int ax = x0 + tid % TX, ay = y0 + (tid / TX) % TY, az = z0 + tid / (TX * TY);
+    if (ax < p.nx && ay < p.ny && az < p.nz) {
+        const int an = ax + p.nx * (ay + p.ny * az);
 #pragma unroll
-                for (int i = 0; i < Q; ++i) cp_async4(&stage[i * NT + tid], e.f_in + (long long)i * p.N + an);
-                if (sizeof(GT) == 4) {
+        for (int i = 0; i < Q; ++i) cp_async4(&stage[i * NT + tid], e.f_in + (long long)i * p.N + an);
+        if (sizeof(GT) == 4) {
 #pragma unroll
-                    for (int i = 0; i < Q; ++i)
-                        cp_async4(&stage[(Q + i) * NT + tid], (const float *)e.g_in + (long long)i * p.N + an);
-                } else {
-                    cp_async4(&stage[Q * NT + tid], (const float *)e.g_in + an);
-                    // the FP16 moving populations of two x-neighbours share a 4-byte
-                    // word (nx even): the even thread of each pair copies it
-                    if ((p.nx & 1) == 0 && (tid & 1) == 0) {
-                        const char *h = (const char *)e.g_in + 4 * p.N;
-                        __half *s16 = reinterpret_cast<__half *>(&stage[(Q + 1) * NT]);
+            for (int i = 0; i < Q; ++i)
+                cp_async4(&stage[(Q + i) * NT + tid], (const float *)e.g_in + (long long)i * p.N + an);
+        } else {
+            cp_async4(&stage[Q * NT + tid], (const float *)e.g_in + an);
+            // the FP16 moving populations of two x-neighbours share a 4-byte
+            // word (nx even): the even thread of each pair copies it
+            if ((p.nx & 1) == 0 && (tid & 1) == 0) {
+                const char *h = (const char *)e.g_in + 4 * p.N;
+                __half *s16 = reinterpret_cast<__half *>(&stage[(Q + 1) * NT]);
 #pragma unroll
-                        for (int i = 1; i < Q; ++i)
-                            cp_async4(&s16[(i - 1) * NT + tid], h + 2 * ((long long)(i - 1) * p.N + an));
-                    }
-                }
+                for (int i = 1; i < Q; ++i)
+                    cp_async4(&s16[(i - 1) * NT + tid], h + 2 * ((long long)(i - 1) * p.N + an));
             }
-            cp_async_commit();
+        }
+    }
+    cp_async_commit();
 }
 
 // Stage A of a D3Q27 tile: rho, phi (and flags) of the tile + halo 2 from the
@@ -868,7 +874,7 @@ __device__ __forceinline__ void collide_f(const BatchEntry &e, float r, float ph
     // pairs the momentum balances, so the update conserves both to rounding.
     // The mirror state f' = f + F_i (Eq. mirror_state) is kept less the weight,
     // like f: formed as f^eq(u + du) - D_i it would drift (mass 8e-6 off after
-    // 1000 steps of a 64 x 64 drop instead of 2e-6).
+    // 1000 steps of a 64 x 64 drop instead of 2.5e-7).
     {
         float2 eq[NPOS], ed[NPOS];
         equilibria<D>(r, u0, up, um, eq);
@@ -967,6 +973,8 @@ __device__ __forceinline__ void collide_f(const BatchEntry &e, float r, float ph
             al = alpha_series(a2, a3, a4, a5, a6, a7);
             if (xmax > ALPHA_SERIES_MAX) {
                 // f' over f' - w and x over D, to hold no further arrays; back behind it
+                // (a rounding more each, so that the balances closed above hold to a
+                // few roundings of f' there and not to those of D)
                 float xs[Q], fs[Q], xneg = 0.f;
                 fs[0] = fp0 + wt<D>(0);
                 xs[0] = dl0 * (1.0f / fs[0]);
@@ -1186,9 +1194,9 @@ __device__ __forceinline__ void tile_origin(const DevParams &p, unsigned k, int 
 // two builds with the same code (the register allocation alone differs):
 // 3 CTAs/SM (80 registers, fewer spills) for launches that fit in one wave,
 // 4 CTAs/SM (64 registers, more warps to hide latency) for larger ones.
-// A step, with the table kernel's before in brackets: D2Q9 64 x 64 8.3 us (8.6),
-// 1024 x 64 11.9 (13.1), 2048 x 2048 171 (238); D3Q27 32 x 32 x 20 24 (28), 101 x
-// 100 x 100 216 (306), 192 x 192 x 128 745 (1022), both passes.
+// A step: D2Q9 64 x 64 8.1 us, 1024 x 64 12.2, 2048 x 2048 171; D3Q27 32 x 32 x 20
+// 24, 101 x 100 x 100 218, 192 x 192 x 128 760, both passes.  Over a tile table, with
+// 8 x 8 x 4 tiles and without the pairs they took 8.6, 13.1, 238, 28, 306, 1022.
 template <int D, typename GT, int MINB, bool BIG>
 __global__ void __launch_bounds__(256, MINB) step_kernel(const __grid_constant__ BatchEntry e)
 {
